@@ -112,7 +112,10 @@ typedef struct {
                            9-12 TMA plane ring with two x points per thread (64);
                            the TMA families give bit-identical results */
     int profile;        /* n > 0: time every n-th stencil launch with CUDA events
-                           (1: every launch); 0: no events */
+                           (1: every launch); 0: no events.  2D calls of few shots
+                           run many time steps per launch (tile = 0,
+                           shots_per_cta = 0): each such launch is timed as a whole
+                           and its mean step time counts for every n-th step */
     int use_graphs;     /* reserved, must be 0 (consecutive steps overlap through
                            programmatic dependent launch; whole runs of uneven
                            problems are graphs in fwi_batch_*) */
@@ -143,8 +146,9 @@ typedef struct {
     size_t workspace_bytes;     /* device bytes held by the plan */
     int64_t launches;           /* kernels launched by the last call */
     int64_t updates;            /* grid-point updates in the last call (all kernels) */
-    int64_t fwd_launches;       /* forward stencil launches (incl. recompute) */
-    int64_t adj_launches;       /* adjoint stencil launches */
+    int64_t fwd_launches;       /* forward stencil launches (incl. recompute); time steps
+                                   where one launch runs many of them */
+    int64_t adj_launches;       /* adjoint stencil launches (time steps) */
     double fwd_ms;              /* summed CUDA-event time of the timed forward stencil launches */
     double adj_ms;              /* same for adjoint stencil launches */
     int64_t fwd_points;         /* grid points (interior) x shots of every forward launch, summed */

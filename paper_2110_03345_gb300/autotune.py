@@ -23,7 +23,7 @@ _CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_autotune_cac
 _lock = threading.Lock()
 
 CANDIDATES_2D = [dict(tile=t, shots_per_cta=s) for t in (5, 6, 7, 8) for s in (2, 3, 4, 5, 6, 8)] + \
-                [dict(tile=t) for t in (1, 2, 3, 4)]
+                [dict(tile=t) for t in (0, 1, 2, 3, 4)]
 CANDIDATES_3D = [dict(tile=t) for t in (5, 6, 7, 8, 9, 10, 11, 12)]
 
 

@@ -200,6 +200,7 @@ fwi_status fwi_batch_create(fwi_batch** out, int nprob, const fwi_problem* probs
     it->prob.geom.rec_xyz = it->recxyz.data();
     const size_t left = hbm_budget_bytes ? (hbm_budget_bytes > used ? hbm_budget_bytes - used : 1) : 0;
     FWI_TRY_B(fwi_plan_create(&it->P, &pr.grid, pr.nt, pr.dt, left, stream));
+    it->P->per_step = true;     // the batch's own launches: one per time step
     fwi_options o{};
     o.batch = pr.geom.nshots;   // every shot of the problem in one batch
     o.tile = opt ? opt->tile : 0;                  // 0: the default (TMA-staged) variant

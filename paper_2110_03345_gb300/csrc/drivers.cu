@@ -391,6 +391,22 @@ fwi_status forward_steps(Call& c, int nb, int shot0, const DevTable& src, float*
                          int K_ckpt, float* CK, float* hist2_base) {
   fwi_plan* P = c.P;
   const size_t fs = (size_t)P->L.fstride;
+  if (c.pl.res.on) {   // runs of steps between checkpoints; the state stays in A, Bf
+    for (int n = n0; n < n1;) {
+      const int end = K_ckpt > 0 ? std::min(n1, (n / K_ckpt + 1) * K_ckpt) : n1;
+      if (K_ckpt > 0 && n % K_ckpt == 0) {
+        float* dst = CK + 2 * (size_t)(n / K_ckpt) * fs * c.pl.B;
+        CUDA_TRY(cudaMemcpyAsync(dst, A, fs * nb * sizeof(float), cudaMemcpyDeviceToDevice, P->st));
+        CUDA_TRY(cudaMemcpyAsync(dst + fs * c.pl.B, Bf, fs * nb * sizeof(float),
+                                 cudaMemcpyDeviceToDevice, P->st));
+      }
+      FWI_TRY(res_forward_steps(c, nb, src, A, Bf, n, end,
+                                hist_base ? hist_base + (size_t)(n - hist_n0) * fs * c.pl.B : nullptr,
+                                sample));
+      n = end;
+    }
+    return FWI_OK;
+  }
   StepParams p = base_params(c);
   p.B = nb;
   p.inj_off = src.off;
@@ -559,7 +575,11 @@ fwi_status begin_call(fwi_plan* P, const fwi_model* model, const fwi_geometry* g
   if (c.W.PQ) c.fstate.push_back(c.W.PQ);
   for (float* ph : c.W.PH)
     if (ph) c.fstate.push_back(ph);
-  if (c.pl.tma) {
+  if (c.W.EX) {
+    CUDA_TRY(cudaMemsetAsync(c.W.EX, 0, c.pl.res.ex * 8, P->st));   // (tags start at 1)
+    c.tag = 0;
+  }
+  if (c.pl.tma && !c.pl.res.on) {
     const bool three = P->grid.ndim == 3;
     for (float* buf : {c.W.U0, c.W.U1, c.W.F0, c.W.F1, c.W.KW}) {
       if (!buf) continue;
@@ -622,6 +642,10 @@ fwi_status begin_call(fwi_plan* P, const fwi_model* model, const fwi_geometry* g
   P->ev_used = 0;
   c.D = c.W.D;
   FWI_TRY(prepare_model(c));
+  if (c.W.INV) {
+    cudaError_t e = launch_res_inv(P->L, P->spx, P->spy, c.W.INV, P->st);
+    if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
+  }
   FWI_TRY(prepare_common(c, tabC));
   return FWI_OK;
 }
@@ -650,6 +674,10 @@ fwi_status finish_call(Call& c) {
     CUDA_TRY(cudaEventElapsedTime(&ms, P->ev[i], P->ev[i + 1]));
     if (P->ev_kind[i] == 0) s.fwd_ms += ms;
     else s.adj_ms += ms;
+  }
+  if (c.pl.res.on) {   // whole launches were timed: the mean step time of the steps counted as timed
+    if (c.fwd_launches) s.fwd_ms *= (double)c.fwd_timed / c.fwd_launches;
+    if (c.adj_launches) s.adj_ms *= (double)c.adj_timed / c.adj_launches;
   }
   if (flags[1] & 2) return fail(FWI_ERR_TIMEOUT, "a bounded wait on a TMA copy timed out");
   if (flags[0]) return fail(FWI_ERR_NONFINITE, "non-finite values in the result (unstable run?)");
@@ -803,6 +831,28 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
       c.adj_launches++;
       c.adj_points += (int64_t)nb * P->L.nx * P->L.ny * P->L.nz;
       std::swap(XN, XC);
+    }
+    return FWI_OK;
+  }
+  if (c.pl.res.on) {
+    for (int k = nt - 1; k >= 1;) {
+      const int ki = std::min(k, nt - 2);   // first imaged step (lambda^{nt-1} = 0 has no term)
+      if (ki >= 1) FWI_TRY(ensure_segment(ki));
+      const int lo = (K > 0 && ki >= 1) ? std::max(seg_lo, 1) : 1;
+      FWI_TRY(res_adjoint_steps(c, nb, LA, LB, k, lo, k == ki, ki >= 1 ? hist_at(ki) : nullptr));
+      k = lo - 1;
+    }
+    if (c.Dw) {   // dJ/dq^0 (the launches sampled lambda^{nt-1} .. lambda^1)
+      cudaError_t e = launch_sample_slots(LA, (long long)fs, c.ws_node, c.ws_w, c.ncorner,
+                                          nb * c.geom->nsrc, c.geom->nsrc, c.Dw, 0, P->st);
+      if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
+      c.launches++;
+    }
+    if (nt >= 2) {
+      FWI_TRY(ensure_segment(0));
+      cudaError_t e = launch_image_only(P->L, LA, hist_at(0), c.W.G, nb, c.pl.S, P->st);
+      c.launches++;
+      if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
     }
     return FWI_OK;
   }
@@ -1036,8 +1086,11 @@ fwi_status fwi_misfit_backward_ex(fwi_plan* P, float* grad_m, float* grad_wavele
   const int nsrc = S->geom.nsrc;
   const size_t npt = (size_t)c.pl.B * nsrc;
   void* wbuf = nullptr;
+  Carve wres(nullptr);
   if (st == FWI_OK && grad_wavelet) {
-    const size_t bytes = align_up((size_t)P->nt * npt * 4, 256) + 2 * align_up(npt * c.ncorner * 4, 256);
+    const size_t bytes = align_up((size_t)P->nt * npt * 4, 256) + 2 * align_up(npt * c.ncorner * 4, 256) +
+                         (c.pl.res.on ? 2 * align_up(npt * c.ncorner * 4, 256) +
+                                            align_up((size_t)c.pl.B * (c.pl.res.P + 1) * 4, 256) : 0);
     e = pool_alloc(&wbuf, bytes, P->st, P->device);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -1050,6 +1103,7 @@ fwi_status fwi_misfit_backward_ex(fwi_plan* P, float* grad_m, float* grad_wavele
       float* w = wc.take<float>(npt * c.ncorner);
       c.ws_node = node;
       c.ws_w = w;
+      wres = wc;   // (the resident kernels' lists follow)
     }
   }
   int batch = 0;
@@ -1063,7 +1117,7 @@ fwi_status fwi_misfit_backward_ex(fwi_plan* P, float* grad_m, float* grad_wavele
       if (e != cudaSuccess) st = fail(FWI_ERR_CUDA, cudaGetErrorString(e));
       if (st == FWI_OK)
         st = build_source_sampling(c, shot0, nb, const_cast<int*>(c.ws_node),
-                                   const_cast<float*>(c.ws_w));
+                                   const_cast<float*>(c.ws_w), wres);
     }
     if (st == FWI_OK) st = gradient_adjoint_batch(c, batch, shot0, nb, src);
     if (st == FWI_OK && c.Dw) {
@@ -1086,6 +1140,7 @@ fwi_status fwi_misfit_backward_ex(fwi_plan* P, float* grad_m, float* grad_wavele
   c.Dw = nullptr;
   c.ws_node = nullptr;
   c.ws_w = nullptr;
+  c.wsmp = ResSamples();
   delete_saved(S);
   return st;
 }

@@ -305,6 +305,61 @@ cudaError_t launch_step3d_x2_ext(const StepParams& p, const CUtensorMap& xm, con
                                  const CUtensorMap& hm, int R, bool vd, bool adj, int mode,
                                  cudaStream_t st);
 
+// Parameters of one resident 2D launch (kernels2d_res.cu): `steps` time steps
+// of blockIdx.y = 0 .. nslots-1 shots (slots), P = gx * gy CTAs of 128 x TH
+// points each per shot.  Per-slot arrays start at the launch's first slot.
+struct ResParams {
+  const float* u;        // u^n (lambda^k) and u^{n-1} (lambda^{k+1}) before the launch
+  const float* up;
+  float* u_out;          // the same after it (may be the same buffers)
+  float* up_out;
+  const float* kf;
+  const float* bx;
+  const float* by;
+  const float* spx;
+  const float* spy;
+  const float* inv;      // 1 / (1 + a) per point (launch_res_inv)
+  float* hist;           // forward: h of the first step (or null), the next steps hstride
+                         // apart; adjoint: h of the first imaged step, then backwards
+  float* g;              // adjoint: gradient slots
+  long long hstride;
+  long long fstride;
+  AxisW wx, wy;
+  int sx, nx, ny, ox, oy;
+  int gx, gy, P, TH;
+  int steps;
+  int img0;              // adjoint: first step of the launch that images (0 or 1)
+  int nimg;              // and how many do
+  const int* inj_off;    // injection entries by (slot, CTA), as StepParams, positions in a
+  const int* inj_loc;    // 128-wide tile
+  const int* inj_vidx;
+  const float* inj_w;
+  const float* vals;
+  long long voff, vstep; // offset of the first step's values, and from step to step
+  int nval;              // most entries of one CTA
+  const int* smp_off;    // raw samples of u^n by CTA (per slot smp_slot apart; or null)
+  const int* smp_loc;    // float offset in the staged tile
+  int smp_slot, smp_locslot;
+  float* raw;            // [step][slot][nraw]
+  int nraw;
+  unsigned long long* ex;   // halo exchange words [slot][CTA][parity][cell][4]
+  unsigned tag0;            // tags of this launch: tag0 + 1 .. tag0 + steps
+  int* flags;
+};
+// ph phases per step, ry rows per thread and phase, nty thread rows (TH = ph * ry * nty;
+// (ph, ry) = (1, 1), (2, 1) or (2, 2))
+cudaError_t launch_res2d(const ResParams& p, int R, bool vd, bool adj, int ph, int ry, int nty, int nslots,
+                         cudaStream_t st);
+size_t res2d_smem(int R, bool vd, bool adj, int TH, int nval);
+int res2d_warps();   // thread rows at most
+int res2d_cells(int R, int TH);   // float4 cells of one CTA's edges (one parity)
+cudaError_t launch_res_inv(const Layout& L, const float* spx, const float* spy, float* inv, cudaStream_t st);
+// out[n out_step + s out_slot + r] = sum_c w raw[n][s][node] for npt points of nc nodes per
+// slot (tables slot_nodes apart; 0: shared), grp lanes per point as sample_receivers
+cudaError_t launch_res_combine(const float* raw, int nraw, int nslots, int steps, const int* node,
+                               const float* w, int slot_nodes, int npt, int nc, int grp, float* out,
+                               long long out_step, long long out_slot, cudaStream_t st);
+
 // Auxiliary kernels (aux_kernels.cu)
 cudaError_t launch_model_prep(const Layout& L, const float* vp, const float* rho, double dt,
                               int param, float* kf, float* lnr, unsigned int* stats,

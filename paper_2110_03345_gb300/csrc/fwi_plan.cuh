@@ -82,6 +82,7 @@ struct fwi_plan {
   size_t ev_used = 0;
   fwi::SavedGrad* saved = nullptr;  // state kept by fwi_misfit_forward for fwi_misfit_backward
   bool fixed_memory = false;   // buffers supplied by the caller: never allocate
+  bool per_step = false;       // one launch per time step always (the problems of a batch)
   ~fwi_plan() { fwi::delete_saved(saved); }
 };
 
@@ -166,6 +167,18 @@ struct Scheme {
   int model_fields() const { return att >= 0 ? 1 : 0; }  // attenuation coefficient
 };
 
+// Resident 2D launches (kernels2d_res.cu): P = gx * gy CTAs per shot, tiles of
+// 128 x TH points (TH = ph * ry * nty), conc shots side by side.
+struct ResPlan {
+  bool on = false;
+  int gx = 0, gy = 0, ph = 1, ry = 1, nty = 1, TH = 0, P = 0, conc = 1;
+  int nval = 0;         // most injection entries of one CTA
+  int chunk = 1;        // steps per launch at most while samples are taken
+  size_t raw = 0;       // floats of the raw sample buffer
+  size_t ex = 0;        // 8-byte words of the halo exchange
+  size_t inv = 0;       // floats of the sponge's 1 / (1 + a)
+};
+
 // Workspace plan for one call.
 struct Plan {
   int B = 1;            // slots
@@ -181,6 +194,7 @@ struct Plan {
   int nbatches = 1;
   size_t bytes = 0;
   Scheme sc;            // extended scheme (then tma, x2 = false, S = 1, tile = 0)
+  ResPlan res;          // resident launches (then S = 1)
 };
 
 // Per-call device state carved out of the arena.
@@ -196,6 +210,18 @@ struct Work {
   float *PH[3] = {nullptr, nullptr, nullptr}, *PHB[3] = {nullptr, nullptr, nullptr};
   double* partials = nullptr;
   int npartials = 0;
+  unsigned long long* EX = nullptr;   // resident launches: halo exchange, raw samples
+  float* RAW = nullptr;
+  float* INV = nullptr;
+};
+
+// Raw sampling lists of the resident kernels: each CTA's nodes, and where
+// each point's nodes land in a step's raw row.
+struct ResSamples {
+  const int* off = nullptr;
+  const int* loc = nullptr;
+  const int* pos = nullptr;
+  int nraw = 0;
 };
 
 struct Call {
@@ -232,6 +258,9 @@ struct Call {
   float* Dw = nullptr;
   const int* ws_node = nullptr;   // [B * nsrc][ncorner] node of each source corner
   const float* ws_w = nullptr;    // its weight / cell volume
+  ResSamples rsmp;                // resident launches: receivers (all slots alike)
+  ResSamples wsmp;                // sources of a batch's slots (dJ/dq)
+  unsigned tag = 0;               // last exchange tag used by this call
 };
 
 // State kept between fwi_misfit_forward and fwi_misfit_backward.
@@ -275,6 +304,7 @@ size_t fixed_bytes(const fwi_plan* P, const fwi_geometry* g, bool vd, int B, con
 fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc);
 fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
                        bool split = false, const Scheme& sc = Scheme());
+int shot_group(const fwi_plan* P, int shape, int B);
 void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Carve& C, Work& W);
 
 // ---- tables.cu: interpolation and injection tables
@@ -298,6 +328,21 @@ fwi_status upload_table(fwi_plan* P, const HostTable& H, Carve& C, DevTable& D);
 fwi_status build_source_table(Call& c, int shot0, int nb, Carve& C, DevTable& D);
 fwi_status prepare_common(Call& c, Carve& tabC);
 size_t tables_bound(const fwi_plan* P, const fwi_geometry* g, const Plan& pl);
+
+// Tile geometry of a call's injection tables.
+TileGeo call_geo(const fwi_plan* P, const Plan& pl);
+
+// ---- resident.cu: on-chip 2D runs
+bool res_eligible(const fwi_plan* P, bool grad, int B, const Scheme& sc);
+size_t res_buffers(const fwi_plan* P, const fwi_geometry* g, int B);   // device bytes, B shots at most
+void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, int B, const Scheme& sc,
+                ResPlan* out);
+fwi_status res_sample_table(Call& c, const std::vector<int>& nodes3, int slots, Carve& C, ResSamples* out);
+fwi_status res_forward_steps(Call& c, int nb, const DevTable& src, float* A, float* Bf, int n0, int n1,
+                             float* hist, bool sample);
+// adjoint steps k = k0 .. k1 (down); hist: h of step k0, or of k0 - 1 when k0 is not imaged
+fwi_status res_adjoint_steps(Call& c, int nb, float* LA, float* LB, int k0, int k1, bool image_first,
+                             float* hist);
 
 // ---- fwi_noalloc.cu
 fwi_status check_on_device(const void* ptr, const char* name, int dev);
@@ -337,6 +382,6 @@ fwi_status gradient_forward_batch(Call& c, int j, int shot0, int nb, const DevTa
                                   const float* observed, float* traces_opt);
 fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTable& src);
 fwi_status gradient_finish(Call& c, int batches, double* misfit, float* grad_m);
-fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float* d_w);
+fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float* d_w, Carve res);
 
 }  // namespace fwi

@@ -340,15 +340,27 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc) {
   return FWI_OK;
 }
 
-fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
-                       bool split, const Scheme& sc) {
+// Shots per CTA of the 2D per-step kernels for B shots: six share a tile's
+// model loads and gradient update; at least four waves of CTAs (two resident
+// per SM) keep the SMs balanced.
+int shot_group(const fwi_plan* P, int shape, int B) {
+  const int T = tile_geo(P, shape, true).ntiles();
+  int S = std::min(B, 6);
+  while (S > 1 && (long long)T * ((B + S - 1) / S) < 8LL * P->nsm) --S;
+  return S;
+}
+
+static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad,
+                                 Plan& out, bool split, const Scheme& sc, bool resident) {
   const int ns = g->nshots;
   const size_t budget = P->budget;
   const int K_auto = std::max(2, (int)std::ceil(std::sqrt(2.0 * std::max(P->nt, 2))));
   const long long N = (long long)P->L.nx * P->L.ny * P->L.nz;
   const int B_fill = (int)std::max(1LL, (8LL << 20) / std::max(N, 1LL));  // slots that fill the GPU
+  // resident 2D launches hold exchange and sample buffers besides
+  const size_t res_bytes = resident ? res_buffers(P, g, P->opt.batch > 0 ? std::min(P->opt.batch, ns) : ns) : 0;
   auto fit = [&](int K) {
-    size_t fixed = fixed_bytes(P, g, vd, ns, sc);
+    size_t fixed = fixed_bytes(P, g, vd, ns, sc) + res_bytes;
     size_t per = slot_bytes(P, g, grad, K, sc);
     if (split) {
       // nbatches * B <= ns + B - 1 shots of kept state
@@ -404,22 +416,28 @@ fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool g
   out.split = split;
   out.nbatches = (ns + B - 1) / B;
   out.S = 1;
-  if (out.tma && P->grid.ndim == 2) {   // the 3D kernels take one shot per CTA
-    if (P->opt.shots_per_cta > 0) {
-      out.S = std::min(P->opt.shots_per_cta, B);
-    } else {
-      // six shots share a tile's model loads and gradient update; at least
-      // four waves of CTAs (two resident per SM) keep the SMs balanced
-      const int T = tile_geo(P, out.shape, true).ntiles();
-      int S = std::min(B, 6);
-      while (S > 1 && (long long)T * ((B + S - 1) / S) < 8LL * P->nsm) --S;
-      out.S = S;
-    }
+  out.res = ResPlan();
+  if (resident) choose_res(P, g, vd, grad, B, sc, &out.res);
+  if (out.res.on) {
+    // (each shot has its own gradient slot)
+  } else if (out.tma && P->grid.ndim == 2) {   // the 3D kernels take one shot per CTA
+    out.S = P->opt.shots_per_cta > 0 ? std::min(P->opt.shots_per_cta, B) : shot_group(P, out.shape, B);
   }
-  out.bytes = fixed_bytes(P, g, vd, B, sc) + (size_t)B * slot_bytes(P, g, grad, K, sc);
+  out.bytes = fixed_bytes(P, g, vd, B, sc) + res_bytes + (size_t)B * slot_bytes(P, g, grad, K, sc);
   if (split)
-    out.bytes = fixed_bytes(P, g, vd, B, sc) + (size_t)B * split_slot_bytes(P, K, sc) +
+    out.bytes = fixed_bytes(P, g, vd, B, sc) + res_bytes + (size_t)B * split_slot_bytes(P, K, sc) +
                 (size_t)out.nbatches * B * persist_bytes_per_shot(P, g, K, sc) + (4u << 20);
+  return FWI_OK;
+}
+
+// The plan with resident launches where the budget holds their buffers and
+// leaves the history mode as it is; else one launch per step.
+fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
+                       bool split, const Scheme& sc) {
+  FWI_TRY(choose_plan_as(P, g, vd, grad, out, split, sc, false));
+  if (!res_eligible(P, grad, out.B, sc)) return FWI_OK;
+  Plan res;
+  if (choose_plan_as(P, g, vd, grad, res, split, sc, true) == FWI_OK && res.res.on && res.K == out.K) out = res;
   return FWI_OK;
 }
 
@@ -438,6 +456,11 @@ void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Car
   if (sc.t4) W.D2Q = C.take<float>((size_t)g->nshots * g->nsrc * P->nt);
   W.npartials = misfit_blocks(B, g->nrec, P->nt);
   W.partials = C.take<double>(W.npartials);
+  if (pl.res.on) {
+    W.EX = C.take<unsigned long long>(pl.res.ex);
+    W.RAW = C.take<float>(pl.res.raw);
+    W.INV = C.take<float>(pl.res.inv);
+  }
   W.U0 = C.take<float>(fs * B);
   W.U1 = C.take<float>(fs * B);
   if (sc.t4) W.KW = C.take<float>(fs * B);

@@ -144,6 +144,19 @@ TileGeo tile_geo(const fwi_plan* P, int tile, bool tma, bool x2, bool ext) {
   return T;
 }
 
+TileGeo call_geo(const fwi_plan* P, const Plan& pl) {
+  if (pl.res.on) {
+    TileGeo T{};
+    T.gx = pl.res.gx;
+    T.gy = pl.res.gy;
+    T.nzc = T.zc = 1;
+    T.tx = TILE_X;
+    T.ty = pl.res.TH;
+    return T;
+  }
+  return tile_geo(P, pl.shape, pl.tma, pl.x2, pl.sc.ext() && !pl.tma);
+}
+
 void add_entry(std::vector<Entry>& E, const TileGeo& T, int slot, const int* node, int vidx,
                float w) {
   const int x = node[0], y = node[1], z = node[2];
@@ -237,14 +250,15 @@ fwi_status build_source_table(Call& c, int shot0, int nb, Carve& C, DevTable& D)
         add_entry(E, c.T, b, &ps.node[3 * q], (s * g->nsrc + k) * P->nt, (float)(ps.w[q] / dV));
     }
   }
-  const HostTable H = bucket(E, c.pl.B * c.T.ntiles(), P->grid.ndim == 2 ? c.T.ty : 0, c.T.tx);
+  const HostTable H = bucket(E, c.pl.B * c.T.ntiles(),
+                             P->grid.ndim == 2 && !c.pl.res.on ? c.T.ty : 0, c.T.tx);
   return upload_table(P, H, C, D);
 }
 
 // Sampling table of the sources of shots shot0 .. shot0+nb-1: per (slot,
 // source) point its corner nodes and weight / cell volume (the transpose of
 // the injection, so that sampling an adjoint field there gives dJ/dq).
-fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float* d_w) {
+fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float* d_w, Carve res) {
   fwi_plan* P = c.P;
   const fwi_geometry* g = c.geom;
   const int nd = P->grid.ndim;
@@ -252,6 +266,7 @@ fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float*
   for (int a = 0; a < nd; ++a) dV *= P->h[a];
   std::vector<int> node((size_t)nb * g->nsrc * c.ncorner, 0);
   std::vector<float> w(node.size(), 0.f);
+  std::vector<int> node3(c.pl.res.on ? 3 * node.size() : 0);
   PointSt ps;
   for (int b = 0; b < nb; ++b)
     for (int k = 0; k < g->nsrc; ++k) {
@@ -261,8 +276,11 @@ fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float*
       for (int q = 0; q < ps.n; ++q) {
         node[pt * c.ncorner + q] = (int)node_index(P->L, &ps.node[3 * q]);
         w[pt * c.ncorner + q] = (float)(ps.w[q] / dV);
+        if (c.pl.res.on)
+          for (int a = 0; a < 3; ++a) node3[3 * (pt * c.ncorner + q) + a] = ps.node[3 * q + a];
       }
     }
+  if (c.pl.res.on) FWI_TRY(res_sample_table(c, node3, c.pl.B, res, &c.wsmp));
   // pageable sources: the copies have staged them when cudaMemcpyAsync returns
   CUDA_TRY(cudaMemcpyAsync(d_node, node.data(), node.size() * 4, cudaMemcpyHostToDevice, P->st));
   CUDA_TRY(cudaMemcpyAsync(d_w, w.data(), w.size() * 4, cudaMemcpyHostToDevice, P->st));
@@ -277,10 +295,11 @@ fwi_status prepare_common(Call& c, Carve& tabC) {
   const fwi_geometry* g = c.geom;
   const int nd = P->grid.ndim;
   c.ncorner = interp_nodes(P->opt.interp, nd);
-  c.T = tile_geo(P, c.pl.shape, c.pl.tma, c.pl.x2, c.pl.sc.ext() && !c.pl.tma);
+  c.T = call_geo(P, c.pl);
   // receiver sampling table
   std::vector<int> node((size_t)g->nrec * c.ncorner);
   std::vector<float> w((size_t)g->nrec * c.ncorner);
+  std::vector<int> node3(c.pl.res.on ? 3 * node.size() : 0);
   std::vector<Entry> E;
   PointSt ps;
   for (int r = 0; r < g->nrec; ++r) {
@@ -289,6 +308,8 @@ fwi_status prepare_common(Call& c, Carve& tabC) {
     for (int q = 0; q < ps.n; ++q) {
       node[(size_t)r * c.ncorner + q] = (int)node_index(P->L, &ps.node[3 * q]);
       w[(size_t)r * c.ncorner + q] = (float)ps.w[q];
+      if (c.pl.res.on)
+        for (int a = 0; a < 3; ++a) node3[3 * ((size_t)r * c.ncorner + q) + a] = ps.node[3 * q + a];
     }
     if (c.pl.gradient)
       for (int b = 0; b < c.pl.B; ++b)
@@ -303,19 +324,22 @@ fwi_status prepare_common(Call& c, Carve& tabC) {
   c.smp_node = dn;
   c.smp_w = dw;
   if (c.pl.gradient) {
-    const HostTable H = bucket(E, c.pl.B * c.T.ntiles(), nd == 2 ? c.T.ty : 0, c.T.tx);
+    const HostTable H = bucket(E, c.pl.B * c.T.ntiles(), nd == 2 && !c.pl.res.on ? c.T.ty : 0, c.T.tx);
     FWI_TRY(upload_table(P, H, tabC, c.rec_tab));
   }
+  if (c.pl.res.on) FWI_TRY(res_sample_table(c, node3, 1, tabC, &c.rsmp));
   return FWI_OK;
 }
 
 size_t tables_bound(const fwi_plan* P, const fwi_geometry* g, const Plan& pl) {
-  const TileGeo T = tile_geo(P, pl.shape, pl.tma, pl.x2, pl.sc.ext() && !pl.tma);
+  const TileGeo T = call_geo(P, pl);
   const int nc = interp_nodes(P->opt.interp, P->grid.ndim);
   const size_t nb = (size_t)pl.B * T.ntiles() + 1;
   const size_t src = (size_t)pl.B * g->nsrc * nc;
   const size_t rec = (size_t)g->nrec * nc;
-  const size_t rows = P->grid.ndim == 2 ? nb * (T.ty + 1) * 4 * 2 + 2 * 256 : 0;   // per-row ranges
+  // per-row ranges, or the resident kernels' sampling lists
+  const size_t rows = pl.res.on ? rec * 8 + nb * 4 + 3 * 256
+                      : P->grid.ndim == 2 ? nb * (T.ty + 1) * 4 * 2 + 2 * 256 : 0;
   return 8 * 256 + nb * 4 * 2 + (src + 1) * 12 + rec * 8 + (pl.gradient ? rec * pl.B * 12 + 4096 : 0) +
          4096 * 4 + rows;
 }
