@@ -190,6 +190,7 @@ struct Plan {
   bool tma = false;     // TMA-staged kernels (2D: shots looped inside a CTA)
   bool x2 = false;      // 3D: two x points per thread (variants 9-12)
   int S = 1;            // shots per CTA; gradient slot of shot s is s / S
+  int zc = 0;           // 3D: planes per CTA (0: the variant's)
   bool split = false;   // forward and adjoint in separate calls: keep every batch's state
   int nbatches = 1;
   size_t bytes = 0;
@@ -305,6 +306,7 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc);
 fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
                        bool split = false, const Scheme& sc = Scheme());
 int shot_group(const fwi_plan* P, int shape, int B);
+int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, int B);
 void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Carve& C, Work& W);
 
 // ---- tables.cu: interpolation and injection tables

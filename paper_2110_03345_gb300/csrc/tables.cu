@@ -154,7 +154,12 @@ TileGeo call_geo(const fwi_plan* P, const Plan& pl) {
     T.ty = pl.res.TH;
     return T;
   }
-  return tile_geo(P, pl.shape, pl.tma, pl.x2, pl.sc.ext() && !pl.tma);
+  TileGeo T = tile_geo(P, pl.shape, pl.tma, pl.x2, pl.sc.ext() && !pl.tma);
+  if (pl.zc > 0) {
+    T.zc = pl.zc;
+    T.nzc = (P->L.nz + T.zc - 1) / T.zc;
+  }
+  return T;
 }
 
 void add_entry(std::vector<Entry>& E, const TileGeo& T, int slot, const int* node, int vidx,
