@@ -328,8 +328,24 @@ fwi_status ext_step(Call& c, const StepParams& p_in, bool adj) {
     }
     c.launches += 2;
   } else {
+    e = cudaSuccess;
+    if (c.pl.sc.ring && adj) {   // lap(att lambda^k) and its change since the step before
+      StepParams a = p;
+      a.x = c.W.KW;
+      a.out = c.W.LC;
+      a.inj_off = nullptr;
+      a.hist = nullptr;
+      a.hist2 = nullptr;
+      a.image = 0;
+      const CUtensorMap* xm = find_map(c, c.W.KW);
+      e = xm ? launch_step3d_x2_ext(a, *xm, *xm, *xm, *xm, *xm, *xm, *xm, P->R, false, false, EXT_LC, P->st)
+             : cudaErrorInvalidValue;
+      c.launches++;
+      p.hist2 = c.W.LC;
+      p.out = c.W.KW;   // att lambda^{k-1}
+    }
     p.x = p.u;
-    e = ext_pass(c, p, adj, c.pl.sc.att == 0 ? EXT_ATT0 : EXT_ATT2);
+    if (e == cudaSuccess) e = ext_pass(c, p, adj, c.pl.sc.att == 0 ? EXT_ATT0 : EXT_ATT2);
     c.launches++;
   }
   if (e != cudaSuccess) return fail(FWI_ERR_CUDA, std::string("stencil launch: ") + cudaGetErrorString(e));
@@ -744,6 +760,7 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
   CUDA_TRY(cudaMemsetAsync(LA, 0, fs * nb * sizeof(float), P->st));
   CUDA_TRY(cudaMemsetAsync(LB, 0, fs * nb * sizeof(float), P->st));
   if (c.W.QA) CUDA_TRY(cudaMemsetAsync(c.W.QA, 0, fs * nb * sizeof(float), P->st));
+  if (c.pl.sc.ring) CUDA_TRY(cudaMemsetAsync(c.W.KW, 0, fs * nb * sizeof(float), P->st));   // att lambda = 0
   const bool ext = c.pl.sc.ext();
   const size_t cm = (size_t)c.pl.sc.ckpt_fields();
   StepParams p = base_params(c);

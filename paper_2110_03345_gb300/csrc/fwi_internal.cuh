@@ -161,6 +161,8 @@ enum ExtMode {
   EXT_T4 = 1,    // F = x + k (L x + s) / 12, update     (4th order, second pass)
   EXT_ATT0 = 2,  // leapfrog with per-point damping alpha0 vp dt   (y = 0)
   EXT_ATT2 = 3,  // leapfrog with the Laplacian-difference term     (y = 2)
+  EXT_LC = 4,    // y = 2 adjoint on the 3D plane ring, first pass: out = lap x - q, q = lap x
+                 // (x = att lambda, written by the step before it)
 };
 constexpr int EXT_TX2 = 128, EXT_TX = 32, EXT_TY2 = 16, EXT_TY3 = 8, EXT_ZC = 32;
 // Perfectly matched layer passes (kernels_pml.cu), same tiles as the extended

@@ -153,6 +153,7 @@ struct Scheme {
   bool t4 = false;   // fourth order in time (options.time_order == 4)
   int att = -1;      // attenuation power y (0 or 2), -1 for none
   bool pml = false;  // perfectly matched layer instead of the sponge (options.boundary == 1)
+  bool ring = false; // y = 2 in 3D on the plane ring (two more fields per slot in gradients)
   int ndim = 2;
   bool ext() const { return t4 || att >= 0 || pml; }
   // PML state besides u^n, u^{n-1}: q (3D) and one phi per axis
@@ -162,8 +163,8 @@ struct Scheme {
     return 2 + (att == 2 ? 1 : 0) + pml_state();
   }
   int fwd_slot_fields() const { return (t4 ? 1 : 0) + (att == 2 ? 1 : 0) + pml_state(); }
-  // adjoint: lap state (y = 2); c, qbar (3D) and the phi adjoints (PML)
-  int adj_slot_fields() const { return (att == 2 ? 1 : 0) + (pml ? 1 + pml_state() : 0); }
+  // adjoint: lap state (y = 2), att lambda and its Laplacian's change (ring); c, qbar (3D) and the phi adjoints (PML)
+  int adj_slot_fields() const { return (att == 2 ? 1 : 0) + (ring ? 2 : 0) + (pml ? 1 + pml_state() : 0); }
   int model_fields() const { return att >= 0 ? 1 : 0; }  // attenuation coefficient
 };
 
@@ -206,6 +207,7 @@ struct Work {
   // extended schemes: attenuation coefficient, k w scratch, Laplacian states
   // (forward, adjoint), second history field, second time difference of the wavelets
   float *ATT = nullptr, *KW = nullptr, *QF = nullptr, *QA = nullptr, *H2 = nullptr, *D2Q = nullptr;
+  float* LC = nullptr;   // y = 2 adjoint on the plane ring (KW then holds att lambda)
   // PML: q and phi (forward), c, qbar and the phi adjoints (adjoint)
   float *PQ = nullptr, *PC = nullptr, *PQB = nullptr;
   float *PH[3] = {nullptr, nullptr, nullptr}, *PHB[3] = {nullptr, nullptr, nullptr};

@@ -1,10 +1,14 @@
 // 3D step kernels of the extended schemes of Sec. 2.4 on the two-point
 // TMA-staged plane ring of the leapfrog (step3d_x2.cuh): the fourth-order
-// time scheme's two passes (EXT_KW, EXT_T4) and the y = 0 attenuation term
-// (EXT_ATT0), forward and adjoint, with the arithmetic of kernels_ext.cu.
-// The plane ring holds the pass's stencil input (u^n, lambda^k, or the
-// k w / k L^T lambda scratch); 64 x 8 columns of 32-plane chunks, one shot
-// per CTA.
+// time scheme's two passes (EXT_KW, EXT_T4) and the attenuation terms (y = 0:
+// EXT_ATT0; y = 2: EXT_ATT2, in the adjoint after EXT_LC).  The plane ring
+// holds the pass's stencil input (u^n, lambda^k, the k w / k L^T lambda scratch,
+// or att lambda); 64 x 8 columns in z chunks, one shot per CTA.
+//
+// The y = 2 adjoint needs lap(att lambda) beside L^T lambda.  A second ring and
+// queue for the product would leave one CTA per SM, so each step also writes
+// att lambda^{k-1} and a Laplacian pass without density terms (EXT_LC) runs
+// ahead of the next one.
 #include "step3d_x2.cuh"
 
 namespace fwi {
@@ -38,6 +42,7 @@ cudaError_t launch_mode3(const StepParams& p, const CUtensorMap* const* m, int m
   switch (mode) {
     case EXT_KW: return launch_e3<R, VD, ADJ, EXT_KW>(p, m, st);
     case EXT_T4: return launch_e3<R, VD, ADJ, EXT_T4>(p, m, st);
+    case EXT_ATT2: return launch_e3<R, VD, ADJ, EXT_ATT2>(p, m, st);
     default: return launch_e3<R, VD, ADJ, EXT_ATT0>(p, m, st);
   }
 }
@@ -49,8 +54,9 @@ cudaError_t launch_step3d_x2_ext(const StepParams& p, const CUtensorMap& xm, con
                                  const CUtensorMap& kfm, const CUtensorMap& gm,
                                  const CUtensorMap& hm, int R, bool vd, bool adj, int mode,
                                  cudaStream_t st) {
-  if (mode != EXT_KW && mode != EXT_T4 && mode != EXT_ATT0) return cudaErrorInvalidValue;
   const CUtensorMap* m[7] = {&xm, &bxm, &bym, &upm, &kfm, &gm, &hm};
+  if (mode == EXT_LC)
+    return R == 4 ? launch_e3<4, false, false, EXT_LC>(p, m, st) : launch_e3<5, false, false, EXT_LC>(p, m, st);
   if (R == 4) {
     if (vd) return adj ? launch_mode3<4, true, true>(p, m, mode, st) : launch_mode3<4, true, false>(p, m, mode, st);
     return adj ? launch_mode3<4, false, true>(p, m, mode, st) : launch_mode3<4, false, false>(p, m, mode, st);

@@ -422,10 +422,10 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
     // TMA shot-loop kernels of 128 x 16 tiles (variant 6), otherwise one
     // shot per CTA (kernels_ext.cu, kernels_pml.cu)
     // in 3D the two-point plane-ring kernels take the fourth-order scheme and
-    // the y = 0 term (variant 12); y = 2 and the PML keep kernels_ext.cu /
-    // kernels_pml.cu
+    // the attenuation (variant 12; y = 2 where its two fields fit); the PML
+    // keeps kernels_pml.cu
     const bool tma2 = P->grid.ndim == 2 && !sc.pml;
-    const bool x2 = P->grid.ndim == 3 && !sc.pml && (sc.t4 || sc.att == 0);
+    const bool x2 = P->grid.ndim == 3 && !sc.pml && (sc.t4 || sc.att == 0 || sc.ring);
     out.tile = tma2 ? 6 : (x2 ? 12 : 0);
     out.shape = tma2 ? 1 : (x2 ? 3 : 0);
     out.tma = tma2 || x2;
@@ -466,6 +466,16 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
 fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
                        bool split, const Scheme& sc) {
   FWI_TRY(choose_plan_as(P, g, vd, grad, out, split, sc, false));
+  if (P->grid.ndim == 3 && sc.att == 2 && !P->fixed_memory) {
+    // the plane ring's two fields must not change what fits (the noalloc
+    // scratch and tight budgets keep the one-point kernels)
+    Scheme ring = sc;
+    ring.ring = true;
+    Plan alt;
+    if (choose_plan_as(P, g, vd, grad, alt, split, ring, false) == FWI_OK && alt.B == out.B && alt.K == out.K)
+      out = alt;
+    return FWI_OK;
+  }
   if (!res_eligible(P, grad, out.B, sc)) return FWI_OK;
   Plan res;
   if (choose_plan_as(P, g, vd, grad, res, split, sc, true) == FWI_OK && res.res.on && res.K == out.K) out = res;
@@ -505,6 +515,10 @@ void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Car
   if (pl.gradient) {
     W.G = C.take<float>(fs * B);
     if (sc.att == 2) W.QA = C.take<float>(fs * B);
+    if (sc.ring) {
+      W.KW = C.take<float>(fs * B);
+      W.LC = C.take<float>(fs * B);
+    }
     if (sc.pml) {
       W.PC = C.take<float>(fs * B);
       if (P->grid.ndim == 3) W.PQB = C.take<float>(fs * B);

@@ -1,6 +1,6 @@
 // The two-point TMA-staged 3D step kernel (kernels3d_x2.cu: the leapfrog;
-// kernels3d_x2_ext.cu: the fourth-order time scheme's passes and the y = 0
-// attenuation term of Sec. 2.4 on the same plane ring).
+// kernels3d_x2_ext.cu: the fourth-order time scheme's passes and the
+// attenuation terms of Sec. 2.4 on the same plane ring).
 #pragma once
 
 #include "fwi_internal.cuh"
@@ -47,10 +47,11 @@ struct GeoX2 {
   static constexpr int NOS = 4;             // operand stages: two loop trips
 };
 
-// MODE: X2_LEAP the leapfrog, or EXT_KW / EXT_T4 / EXT_ATT0 (fwi_internal.cuh)
-// with the arithmetic of kernels_ext.cu: the plane ring holds the stencil
-// input (u^n, lambda^k, or the k w / k L^T lambda scratch), and the update
-// writes k (L x + s) (EXT_KW) or the fourth-order / attenuating update.
+// MODE: X2_LEAP the leapfrog, or an extended scheme (ExtMode, fwi_internal.cuh):
+// the plane ring holds the stencil input (u^n, lambda^k, the k w / k L^T lambda
+// scratch, or att lambda), and the update writes k (L x + s) (EXT_KW), the
+// Laplacian and its change since the previous step (EXT_LC), or the
+// fourth-order / attenuating update.
 constexpr int X2_LEAP = -1;
 constexpr float X2_INV12 = 1.f / 12.f;   // the fourth-order scheme's 1/12, rounded once
 
@@ -79,7 +80,7 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
   constexpr int NOS = G::NOS;
   // operand stages (variable density): [NOS][lambda^{k+1}, k, h, g][BY][TXP]
   // in the adjoint, [NOS][u^{n-1}, k][BY][TXP] in the forward
-  constexpr bool OPS = VD;
+  constexpr bool OPS = VD;                    // (EXT_LC runs without density)
   constexpr int OPN = ADJ ? 4 : 2;            // operand tiles per stage
   float* ops = bring + (PSI ? NBS * G::BSTAGE : 0);
   __shared__ uint64_t bar[NSU];
@@ -216,8 +217,10 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
   const int loc0 = ty * G::TXP + 2 * tx;    // entry location of the own pair in plane lz = 0
 
   constexpr bool KWM = MODE == EXT_KW, T4M = MODE == EXT_T4, A0M = MODE == EXT_ATT0;
-  // (the extended schemes' u^n (lambda^k), k w^k and damping: x[0..2], only
-  // in their instantiations)
+  constexpr bool A2M = MODE == EXT_ATT2, LCM = MODE == EXT_LC;
+  // (the extended schemes' u^n (lambda^k), k w^k and attenuation: x[0..2], only
+  // in their instantiations; y = 2: x[0] the previous Laplacian, in the adjoint
+  // the change of lap(att lambda))
   constexpr int NX = (MODE == X2_LEAP) ? 1 : 3;
   struct Ops {
     float2 uo, kk, hv, gv, bx, by, bz, bzl;
@@ -237,12 +240,14 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
       o.x[0] = *reinterpret_cast<const float2*>(p.u + fo + id);
       if (ADJ && p.image) o.x[1] = __ldcs(reinterpret_cast<const float2*>(p.hist2 + fo + id));
     }
-    if (A0M) o.x[2] = ldg2(p.att + id);
+    if (A0M || A2M) o.x[2] = ldg2(p.att + id);
+    if (LCM || (A2M && !ADJ)) o.x[0] = *reinterpret_cast<const float2*>(p.q + fo + id);
+    if (A2M && ADJ) o.x[0] = *reinterpret_cast<const float2*>(p.hist2 + fo + id);
     if (PSI) {   // lambda^{k+1}, k, h, g come from the operand stages
       o.bzl = ldg2(p.bz + (long long)(pz0 + ii + 2 * R) * p.sxy + col);
       return o;
     }
-    if (!OPS) {   // (OPS: u^{n-1} and k come from the operand stages)
+    if (!OPS && !LCM) {   // (OPS: u^{n-1} and k come from the operand stages)
       o.uo = *reinterpret_cast<const float2*>(p.up + fo + id);
       o.kk = ldg2(p.kf + id);
     }
@@ -313,6 +318,7 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
         float2 acc = __fmul2_rn(ax, bc2(p.ih2[0]));
         acc = __ffma2_rn(ay, bc2(p.ih2[1]), acc);
         acc = __ffma2_rn(az, bc2(p.ih2[2]), acc);
+        const float2 lap2 = acc;   // y = 2: the plain Laplacian
         if (VD && !ADJ) {
           float2 dx = z2, dy = z2, dz = z2;
 #pragma unroll
@@ -418,35 +424,58 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
           const float hvv[2] = {hv.x, hv.y}, h2v[2] = {h22.x, h22.y};
           const float gvv[2] = {gv.x, gv.y}, atv[2] = {at2.x, at2.y};
           const float av[2] = {a.x, a.y};
-          const bool inl[2] = {in0, in1};
+          const float lp[2] = {lap2.x, lap2.y};
+          float ov[2], rv[2], hw[2], gw[2], qv[2];   // out, u^{n+1}, history, gradient, state
 #pragma unroll
           for (int l = 0; l < 2; ++l) {
-            if (!inl[l]) continue;
-            const long long o = fo + idx + l;
+            ov[l] = rv[l] = hw[l] = gw[l] = qv[l] = 0.f;
             if (KWM) {
-              p.out[o] = kv[l] * ac[l];
-              continue;
-            }
-            float r, hval = 0.f;
-            if (T4M) {
+              ov[l] = kv[l] * ac[l];
+            } else if (LCM) {
+              qv[l] = ac[l];
+              ov[l] = ac[l] - ucv[l];
+            } else if (T4M) {
               const float F = fmaf(kv[l] * ac[l], X2_INV12, cn[l]);
-              r = (2.f * ucv[l] - (1.f - av[l]) * uov[l] + F) * __frcp_rn(1.f + av[l]);
-              hval = F;
-            } else {   // A0M
+              rv[l] = (2.f * ucv[l] - (1.f - av[l]) * uov[l] + F) * __frcp_rn(1.f + av[l]);
+              hw[l] = F;
+              gw[l] = gvv[l] - fmaf(cn[l] * h2v[l], X2_INV12, ucv[l] * hvv[l]);
+            } else if (A0M) {
               const float aa = av[l] + atv[l];
               const float hh = kv[l] * ac[l];
-              r = (2.f * cn[l] - (1.f - aa) * uov[l] + hh) * __frcp_rn(1.f + aa);
-              hval = hh - 0.5f * atv[l] * (r - uov[l]);
+              rv[l] = (2.f * cn[l] - (1.f - aa) * uov[l] + hh) * __frcp_rn(1.f + aa);
+              hw[l] = hh - 0.5f * atv[l] * (rv[l] - uov[l]);
+              gw[l] = fmaf(-cn[l], hvv[l], gvv[l]);
+            } else {   // A2M
+              const float dl = ADJ ? ucv[l] : lp[l] - ucv[l];
+              const float hh = kv[l] * (ADJ ? ac[l] + dl : fmaf(atv[l], dl, ac[l]));
+              rv[l] = (2.f * cn[l] - (1.f - av[l]) * uov[l] + hh) * __frcp_rn(1.f + av[l]);
+              hw[l] = hh + 0.5f * kv[l] * atv[l] * dl;
+              gw[l] = fmaf(-cn[l], hvv[l], gvv[l]);
+              qv[l] = lp[l];
+              ov[l] = atv[l] * rv[l];
             }
-            p.up[o] = r;
+          }
+          // the pair's stores, the last one of an odd row by itself
+          auto put = [&](float* f, const float* v, bool stream) {
+            if (in1) {
+              float2* q = reinterpret_cast<float2*>(f + fo + idx);
+              if (stream) __stcs(q, make_float2(v[0], v[1]));
+              else *q = make_float2(v[0], v[1]);
+            } else if (in0) {
+              f[fo + idx] = v[0];
+            }
+          };
+          if (KWM || LCM || (A2M && ADJ)) put(p.out, ov, false);
+          if (LCM || (A2M && !ADJ)) put(p.q, qv, false);
+          if (!KWM && !LCM) {
+            put(p.up, rv, false);
             if (!ADJ) {
               if (p.hist) {
-                __stcs(p.hist + o, hval);
-                if (T4M) __stcs(p.hist2 + o, cn[l]);
+                put(p.hist, hw, true);
+                if (T4M) put(p.hist2, cn, true);
               }
             } else if (p.image) {
-              p.g[o] = T4M ? gvv[l] - fmaf(cn[l] * h2v[l], X2_INV12, ucv[l] * hvv[l])
-                           : fmaf(-cn[l], hvv[l], gvv[l]);
+              put(p.g, gw, false);
             }
           }
           continue;
