@@ -360,13 +360,23 @@ fwi_status ext_step(Call& c, const StepParams& p_in, bool adj) {
   return FWI_OK;
 }
 
-// One PML time step (kernels_pml.cu), counted and timed as one stencil
+// One pass of the PML, and one PML time step, counted and timed as one stencil
 // launch: the u update (u^{n+1} over u^{n-1}, q^{n+1}, h^n), then the phi
 // update from u^{n+1} and q^{n+1}.
+cudaError_t pml_pass(const Call& c, const StepParams& p, int mode) {
+  const fwi_plan* P = c.P;
+  if (P->grid.ndim == 2) return launch_pml2d(p, P->R, c.vd, mode, P->st);
+  const float* ring = mode == PML_A ? c.W.U0 : p.x;
+  const float* row = mode == PML_A ? c.W.PHB[0] : (mode == PML_B && c.vd) ? c.W.bx : c.W.PH[0];
+  const float* col = mode == PML_A ? c.W.PHB[1] : (mode == PML_B && c.vd) ? c.W.by : c.W.PH[1];
+  const CUtensorMap *xm = find_map(c, ring), *rm = find_map(c, row), *cm = find_map(c, col);
+  if (!xm || !rm || !cm) return cudaErrorInvalidValue;
+  return launch_pml3d(p, *xm, *rm, *cm, P->R, c.vd, mode, P->st);
+}
+
 fwi_status pml_step(Call& c, const StepParams& p_in) {
   fwi_plan* P = c.P;
   StepParams p = p_in;
-  const int nd = P->grid.ndim;
   if (p.nrec > 0 && (long long)p.B * p.nrec * p.smp_group > launch_threads(c, p.B)) {
     cudaError_t e = launch_sample(p, P->st);
     if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
@@ -379,14 +389,15 @@ fwi_status pml_step(Call& c, const StepParams& p_in) {
   p.q = c.W.PQ;
   for (int d = 0; d < 3; ++d) p.ph[d] = c.W.PH[d];
   if (prof) FWI_TRY(record_event(P, 0));
-  cudaError_t e = launch_pml(p, nd, P->R, c.vd, PML_U, P->st);
+  p.flags = P->d_flags + 1;
+  cudaError_t e = pml_pass(c, p, PML_U);
   if (e == cudaSuccess) {
     StepParams b = p;
     b.x = p.up;            // u^{n+1}
     b.nrec = 0;
     b.inj_off = nullptr;
     b.hist = nullptr;
-    e = launch_pml(b, nd, P->R, c.vd, PML_PHI, P->st);
+    e = pml_pass(c, b, PML_PHI);
   }
   c.launches += 2;
   if (e != cudaSuccess) return fail(FWI_ERR_CUDA, std::string("PML launch: ") + cudaGetErrorString(e));
@@ -609,6 +620,19 @@ fwi_status begin_call(fwi_plan* P, const fwi_model* model, const fwi_geometry* g
         c.maps.push_back(mi);
       }
     }
+    if (three && c.pl.sc.pml) {
+      // the PML's row (80 x BY) and column (64 x BY + 2R) tiles, k c's planes
+      const int by = tile3_variant(c.pl.shape).by;
+      const struct { float* buf; int bw, bh; } f[5] = {{c.W.PH[0], 80, by}, {c.W.PHB[0], 80, by},
+                                                       {c.W.PH[1], 64, by + 2 * P->R},
+                                                       {c.W.PHB[1], 64, by + 2 * P->R}, {c.W.PC, 0, 0}};
+      for (const auto& t : f) {
+        if (!t.buf) continue;
+        Call::MapEnt m{t.buf, {}};
+        FWI_TRY(make_tensor_map_3d(P, t.buf, c.pl.B, c.pl.shape, true, &m.map, t.bw, t.bh));
+        c.maps.push_back(m);
+      }
+    }
     if (three && c.vd && c.pl.x2) {
       // the two-point variable-density kernels read u^{n-1} (lambda^{k+1}), k
       // and g by TMA in 64 x BY plane tiles
@@ -801,13 +825,13 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
                          bb.H2);
   };
   if (c.pl.sc.pml) {
-    // PML adjoint (kernels_pml.cu): ubar^{n+1} in XN, ubar^n in XC, c^n, qbar,
+    // PML adjoint (kernels_pml.cu, kernels_pml3d.cu): ubar^{n+1} in XN, ubar^n in XC, c^n, qbar,
     // the phi adjoints; ubar^{nt-1} = P^T r^{nt-1}, ubar^{nt-2} = P^T r^{nt-2}
     float* XN = LA;
     float* XC = LB;
     for (float* f : {c.W.PC, c.W.PQB, c.W.PHB[0], c.W.PHB[1], c.W.PHB[2]})
       if (f) CUDA_TRY(cudaMemsetAsync(f, 0, fs * nb * sizeof(float), P->st));
-    const int nd = P->grid.ndim;
+    p.flags = P->d_flags + 1;
     for (int m = 0; m < 2 && nt - 1 - m >= 0; ++m) {
       StepParams pi = p;
       pi.step_off = (long long)(nt - 1 - m) * B * c.geom->nrec;
@@ -827,17 +851,18 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
       pa.q = c.W.PQB;
       for (int d = 0; d < 3; ++d) pa.ph[d] = c.W.PHB[d];
       pa.hist = hist_at(n);
+      pa.hist2 = XC;   // (3D: the first pass adds (2 - e) c there)
       pa.image = 1;
       pa.step_off = (long long)(n - 1) * B * c.geom->nrec;
       if (n < 1) pa.inj_off = nullptr;   // no residual before the record
-      cudaError_t e = launch_pml(pa, nd, P->R, c.vd, PML_A, P->st);
+      cudaError_t e = pml_pass(c, pa, PML_A);
       if (e == cudaSuccess) {
         StepParams pb = p;
         pb.x = c.W.PC;
         pb.up = XC;
         for (int d = 0; d < 3; ++d) pb.ph[d] = c.W.PHB[d];
         pb.inj_off = nullptr;
-        e = launch_pml(pb, nd, P->R, c.vd, PML_B, P->st);
+        e = pml_pass(c, pb, PML_B);
       }
       if (e != cudaSuccess) return fail(FWI_ERR_CUDA, std::string("PML launch: ") + cudaGetErrorString(e));
       c.launches += 2;

@@ -97,7 +97,7 @@ struct StepParams {
   float* q;              // y = 2: Laplacian of the previous step (updated in place)
   float* hist2;          // fourth-order scheme: k w^n (forward store, adjoint read)
   float inj_scale;       // factor on injected values (fourth-order adjoint pass B: 12)
-  // perfectly matched layer (kernels_pml.cu): auxiliary fields phi_x, phi_y,
+  // perfectly matched layer (kernels_pml.cu, kernels_pml3d.cu): auxiliary fields phi_x, phi_y,
   // phi_z (forward) or their adjoints, the time step, the layer width
   float* ph[3];
   float dt;
@@ -165,12 +165,17 @@ enum ExtMode {
                  // (x = att lambda, written by the step before it)
 };
 constexpr int EXT_TX2 = 128, EXT_TX = 32, EXT_TY2 = 16, EXT_TY3 = 8, EXT_ZC = 32;
-// Perfectly matched layer passes (kernels_pml.cu), same tiles as the extended
-// schemes: forward u update, forward phi update, adjoint pass A (the phi and
+// Perfectly matched layer passes (2D: kernels_pml.cu, the extended schemes'
+// tiles; 3D: kernels_pml3d.cu, the plane ring's columns): forward u update, forward phi update, adjoint pass A (the phi and
 // q adjoints into ubar^{n+1}, c^n, imaging), adjoint pass B (L^T(k c) and the
 // phi adjoints).
 enum PmlMode { PML_U = 0, PML_PHI = 1, PML_A = 2, PML_B = 3 };
-cudaError_t launch_pml(const StepParams& p, int ndim, int R, bool vd, int mode, cudaStream_t st);
+cudaError_t launch_pml2d(const StepParams& p, int R, bool vd, int mode, cudaStream_t st);
+// xm: the stencil input's planes (PML_U u^n, PML_PHI u^{n+1}, PML_B k c); rm, cm: row and
+// column tiles (PML_U phi_x, phi_y; PML_A their adjoints; PML_B b_x, b_y).  PML_A: p.up =
+// ubar^{n+1}, p.hist2 = ubar^n, p.out = k c^n.
+cudaError_t launch_pml3d(const StepParams& p, const CUtensorMap& xm, const CUtensorMap& rm,
+                         const CUtensorMap& cm, int R, bool vd, int mode, cudaStream_t st);
 // field[slot][node] += w vals[vidx + step_off] over the buckets of p.B slots
 // (tile geometry tx x ty x zc, gx x gy tiles per plane chunk)
 cudaError_t launch_inject_buckets(const StepParams& p, float* field, int tx, int ty, int zc, int gx,

@@ -425,7 +425,7 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
     // the attenuation (variant 12; y = 2 where its two fields fit); the PML
     // keeps kernels_pml.cu
     const bool tma2 = P->grid.ndim == 2 && !sc.pml;
-    const bool x2 = P->grid.ndim == 3 && !sc.pml && (sc.t4 || sc.att == 0 || sc.ring);
+    const bool x2 = P->grid.ndim == 3 && (sc.pml || sc.t4 || sc.att == 0 || sc.ring);
     out.tile = tma2 ? 6 : (x2 ? 12 : 0);
     out.shape = tma2 ? 1 : (x2 ? 3 : 0);
     out.tma = tma2 || x2;
@@ -445,7 +445,7 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
   out.nbatches = (ns + B - 1) / B;
   out.zc = 0;
   if (P->grid.ndim == 3 && P->opt.tile == 0 && out.x2 && !P->fixed_memory)
-    out.zc = z_chunk(P, tile_geo(P, out.shape, out.tma, out.x2), vd, grad, B);
+    out.zc = z_chunk(P, tile_geo(P, out.shape, out.tma, out.x2), vd || sc.pml, grad, B);
   out.S = 1;
   out.res = ResPlan();
   if (resident) choose_res(P, g, vd, grad, B, sc, &out.res);
