@@ -365,7 +365,10 @@ fwi_status ext_step(Call& c, const StepParams& p_in, bool adj) {
 // update from u^{n+1} and q^{n+1}.
 cudaError_t pml_pass(const Call& c, const StepParams& p, int mode) {
   const fwi_plan* P = c.P;
-  if (P->grid.ndim == 2) return launch_pml2d(p, P->R, c.vd, mode, P->st);
+  if (P->grid.ndim == 2) {
+    if (mode == PML_PHI || mode == PML_A) return launch_pml2d(p, P->R, mode, P->st);
+    return ext_pass(c, p, mode == PML_B, EXT_PML);
+  }
   const float* ring = mode == PML_A ? c.W.U0 : p.x;
   const float* row = mode == PML_A ? c.W.PHB[0] : (mode == PML_B && c.vd) ? c.W.bx : c.W.PH[0];
   const float* col = mode == PML_A ? c.W.PHB[1] : (mode == PML_B && c.vd) ? c.W.by : c.W.PH[1];
@@ -390,6 +393,7 @@ fwi_status pml_step(Call& c, const StepParams& p_in) {
   for (int d = 0; d < 3; ++d) p.ph[d] = c.W.PH[d];
   if (prof) FWI_TRY(record_event(P, 0));
   p.flags = P->d_flags + 1;
+  p.S = c.pl.S;
   cudaError_t e = pml_pass(c, p, PML_U);
   if (e == cudaSuccess) {
     StepParams b = p;
@@ -825,55 +829,85 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
                          bb.H2);
   };
   if (c.pl.sc.pml) {
-    // PML adjoint (kernels_pml.cu, kernels_pml3d.cu): ubar^{n+1} in XN, ubar^n in XC, c^n, qbar,
-    // the phi adjoints; ubar^{nt-1} = P^T r^{nt-1}, ubar^{nt-2} = P^T r^{nt-2}
+    // PML adjoint.  3D (kernels_pml3d.cu): ubar^{n+1} in XN, ubar^n in XC, k c^n in
+    // PC; 2D (kernels_pml.cu): lambda^n in XN, lambda^{n-1} in XC, the layer's share
+    // of ubar in all three.  ubar^{nt-1} = P^T r^{nt-1}, ubar^{nt-2} = P^T r^{nt-2}.
     float* XN = LA;
     float* XC = LB;
+    const bool two = P->grid.ndim == 2;
     for (float* f : {c.W.PC, c.W.PQB, c.W.PHB[0], c.W.PHB[1], c.W.PHB[2]})
       if (f) CUDA_TRY(cudaMemsetAsync(f, 0, fs * nb * sizeof(float), P->st));
     p.flags = P->d_flags + 1;
+    p.S = c.pl.S;
+    for (int d = 0; d < 3; ++d) p.ph[d] = c.W.PHB[d];
+    cudaError_t e = cudaSuccess;
+    auto pass = [&](const StepParams& q, int mode) {
+      if (e == cudaSuccess) e = pml_pass(c, q, mode);
+      c.launches++;
+    };
+    if (two && nt >= 2) {
+      FWI_TRY(make_tensor_map_hist(P, bb.H, B, K == 0 ? std::max(nt - 1, 1) : K, c.pl.shape, &c.hmap));
+      c.hmap_ok = true;
+      StepParams ps = p;   // lambda^{nt-2} = k P^T r^{nt-1} away from the layer
+      ps.x = ps.u = XN;
+      ps.up = XC;
+      ps.image = 0;
+      ps.hist = nullptr;
+      ps.step_off = (long long)(nt - 1) * B * c.geom->nrec;
+      pass(ps, PML_B);
+      std::swap(XN, XC);
+    }
     for (int m = 0; m < 2 && nt - 1 - m >= 0; ++m) {
       StepParams pi = p;
       pi.step_off = (long long)(nt - 1 - m) * B * c.geom->nrec;
-      cudaError_t e = launch_inject_buckets(pi, m == 0 ? XN : XC, c.T.tx, c.T.ty, c.T.zc, c.T.gx,
-                                            c.T.gy, P->st);
-      if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
+      float* f = m == 0 ? XN : (two ? c.W.PC : XC);
+      if (e == cudaSuccess)
+        e = launch_inject_buckets(pi, f, c.T.tx, c.T.ty, c.T.zc, c.T.gx, c.T.gy,
+                                  two ? P->grid.sponge + P->R : 0, P->st);
       c.launches++;
     }
-    for (int n = nt - 2; n >= 0; --n) {
+    for (int n = nt - 2; n >= 0 && e == cudaSuccess; --n) {
       FWI_TRY(ensure_segment(n));
       const bool prof = P->opt.profile > 0 &&
                         (c.fwd_launches + c.adj_launches) % P->opt.profile == 0;
       if (prof) FWI_TRY(record_event(P, 1));
       StepParams pa = p;
       pa.up = XN;
-      pa.out = c.W.PC;
+      pa.out = two ? XC : c.W.PC;
+      pa.hist2 = two ? c.W.PC : XC;
       pa.q = c.W.PQB;
-      for (int d = 0; d < 3; ++d) pa.ph[d] = c.W.PHB[d];
       pa.hist = hist_at(n);
-      pa.hist2 = XC;   // (3D: the first pass adds (2 - e) c there)
-      pa.image = 1;
+      pa.image = two ? n > 0 : 1;        // (2D: lambda^0 images below)
       pa.step_off = (long long)(n - 1) * B * c.geom->nrec;
       if (n < 1) pa.inj_off = nullptr;   // no residual before the record
-      cudaError_t e = pml_pass(c, pa, PML_A);
-      if (e == cudaSuccess) {
+      pass(pa, PML_A);
+      if (!two || n > 0) {
         StepParams pb = p;
-        pb.x = c.W.PC;
+        pb.x = pb.u = two ? XN : c.W.PC;
         pb.up = XC;
-        for (int d = 0; d < 3; ++d) pb.ph[d] = c.W.PHB[d];
-        pb.inj_off = nullptr;
-        e = pml_pass(c, pb, PML_B);
+        if (two) {
+          pb.image = 1;
+          pb.hist = hist_at(n);
+          pb.hstep = (int)((size_t)(pb.hist - bb.H) / (fs * B));
+          pb.step_off = (long long)n * B * c.geom->nrec;
+        } else {
+          pb.inj_off = nullptr;
+        }
+        pass(pb, PML_B);
       }
-      if (e != cudaSuccess) return fail(FWI_ERR_CUDA, std::string("PML launch: ") + cudaGetErrorString(e));
-      c.launches += 2;
       if (prof) {
         FWI_TRY(record_event(P, 1));
         c.adj_timed++;
       }
       c.adj_launches++;
       c.adj_points += (int64_t)nb * P->L.nx * P->L.ny * P->L.nz;
-      std::swap(XN, XC);
+      if (!two || n > 0) std::swap(XN, XC);
     }
+    if (two && nt >= 2 && e == cudaSuccess) {   // imaging term of lambda^0 (slot b / 1: one per shot)
+      e = launch_image_only(P->L, XN, hist_at(0), c.W.G, nb, 1, P->st);
+      c.launches++;
+    }
+    if (e != cudaSuccess) return fail(FWI_ERR_CUDA, std::string("PML launch: ") + cudaGetErrorString(e));
     return FWI_OK;
   }
   if (c.pl.res.on) {
@@ -973,7 +1007,8 @@ fwi_status gradient_adjoint_batch(Call& c, int j, int shot0, int nb, const DevTa
 // `batches` batches (0: none) and finish the call.
 fwi_status gradient_finish(Call& c, int batches, double* misfit, float* grad_m) {
   fwi_plan* P = c.P;
-  const int G = (c.pl.B + c.pl.S - 1) / c.pl.S;   // gradient slots in use
+  // gradient slots in use (the PML's layer passes take one per shot)
+  const int G = c.pl.sc.pml ? c.pl.B : (c.pl.B + c.pl.S - 1) / c.pl.S;
   if (grad_m) {
     cudaError_t e = launch_grad_finalize(P->L, c.W.G, G, 1.0 / (P->dt * P->dt), grad_m, P->d_flags, P->st);
     if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));

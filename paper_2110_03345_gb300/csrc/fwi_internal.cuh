@@ -163,6 +163,8 @@ enum ExtMode {
   EXT_ATT2 = 3,  // leapfrog with the Laplacian-difference term     (y = 2)
   EXT_LC = 4,    // y = 2 adjoint on the 3D plane ring, first pass: out = lap x - q, q = lap x
                  // (x = att lambda, written by the step before it)
+  EXT_PML = 5,   // 2D perfectly matched layer: PML_U, and PML_B with the leapfrog
+                 // adjoint away from the layer (kernels_pml.cu)
 };
 constexpr int EXT_TX2 = 128, EXT_TX = 32, EXT_TY2 = 16, EXT_TY3 = 8, EXT_ZC = 32;
 // Perfectly matched layer passes (2D: kernels_pml.cu, the extended schemes'
@@ -170,16 +172,21 @@ constexpr int EXT_TX2 = 128, EXT_TX = 32, EXT_TY2 = 16, EXT_TY3 = 8, EXT_ZC = 32
 // q adjoints into ubar^{n+1}, c^n, imaging), adjoint pass B (L^T(k c) and the
 // phi adjoints).
 enum PmlMode { PML_U = 0, PML_PHI = 1, PML_A = 2, PML_B = 3 };
-cudaError_t launch_pml2d(const StepParams& p, int R, bool vd, int mode, cudaStream_t st);
+// 2D PML: the points whose float4 (first x: xg, row y) comes within W points of a face.
+__host__ __device__ __forceinline__ bool pml_near(int xg, int y, int W, int nx, int ny) {
+  return y < W || y >= ny - W || xg < W || xg + 4 > nx - W;
+}
+cudaError_t launch_pml2d(const StepParams& p, int R, int mode, cudaStream_t st);   // PML_PHI, PML_A
 // xm: the stencil input's planes (PML_U u^n, PML_PHI u^{n+1}, PML_B k c); rm, cm: row and
 // column tiles (PML_U phi_x, phi_y; PML_A their adjoints; PML_B b_x, b_y).  PML_A: p.up =
 // ubar^{n+1}, p.hist2 = ubar^n, p.out = k c^n.
 cudaError_t launch_pml3d(const StepParams& p, const CUtensorMap& xm, const CUtensorMap& rm,
                          const CUtensorMap& cm, int R, bool vd, int mode, cudaStream_t st);
 // field[slot][node] += w vals[vidx + step_off] over the buckets of p.B slots
-// (tile geometry tx x ty x zc, gx x gy tiles per plane chunk)
+// (tile geometry tx x ty x zc, gx x gy tiles per plane chunk); reach > 0: only those at
+// 2D points near a face (pml_near)
 cudaError_t launch_inject_buckets(const StepParams& p, float* field, int tx, int ty, int zc, int gx,
-                                  int gy, cudaStream_t st);
+                                  int gy, int reach, cudaStream_t st);
 cudaError_t launch_ext(const StepParams& p, int ndim, int R, bool vd, bool adj, int mode,
                        cudaStream_t st);
 // out[i] = q[i+1] - 2 q[i] + q[i-1] along the last axis of rows x nt samples
@@ -276,7 +283,7 @@ cudaError_t launch_step2d_tma(const StepParams& p, const CUtensorMap& map, const
 void tma_box2d(int R, int tile, int* bx, int* by);
 void tma_box2d_interior(int tile, int* bx, int* by);
 // The extended schemes' 2D kernels on the same pipeline (kernels2d_tma_ext.cu):
-// mode = EXT_KW / EXT_T4 / EXT_ATT0 / EXT_ATT2, map = the tensor map of the
+// mode = EXT_KW / EXT_T4 / EXT_ATT0 / EXT_ATT2 / EXT_PML, map = the tensor map of the
 // stencil input p.x for tile shape 1 (128 x 16), um of p.up without halo, hm
 // / h2m of the history fields (read by the adjoint when p.image), ucm of
 // p.u without halo (read by the fourth-order update), p.S shots per CTA.

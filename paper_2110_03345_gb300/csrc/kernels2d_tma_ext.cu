@@ -1,7 +1,8 @@
 // 2D step kernels of the extended schemes of Sec. 2.4 on the TMA-staged
 // shot-loop pipeline of the leapfrog (tma2d_tile.cuh): the fourth-order time
-// scheme's two passes (EXT_KW, EXT_T4) and the attenuating leapfrog (EXT_ATT0,
-// EXT_ATT2), forward and adjoint, with the arithmetic of kernels_ext.cu.
+// scheme's two passes (EXT_KW, EXT_T4), the attenuating leapfrog (EXT_ATT0,
+// EXT_ATT2) and the perfectly matched layer (EXT_PML, with the layer's passes of
+// kernels_pml.cu), forward and adjoint.
 //
 // A CTA of 32 x 16 threads owns a 128 x 16 tile for a group of S shots: the
 // stencil input x of each shot (u^n, lambda^k, or the k w / k L^T lambda
@@ -59,6 +60,7 @@ cudaError_t launch_mode(const StepParams& p, const CUtensorMap* const* maps, int
     case EXT_KW: return launch_e<R, VD, ADJ, EXT_KW>(p, maps, st);
     case EXT_T4: return launch_e<R, VD, ADJ, EXT_T4>(p, maps, st);
     case EXT_ATT0: return launch_e<R, VD, ADJ, EXT_ATT0>(p, maps, st);
+    case EXT_PML: return launch_e<R, VD, ADJ, EXT_PML>(p, maps, st);
     default: return launch_e<R, VD, ADJ, EXT_ATT2>(p, maps, st);
   }
 }

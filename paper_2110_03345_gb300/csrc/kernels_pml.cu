@@ -19,8 +19,18 @@
 //            g -= (k c^n) h^n   (the imaging condition of Sec. 2.2, Eq. 8);
 //   PML_B:   ubar^n += (2 - e) c^n + L^T(k c^n),
 //            phibar_j^n = p_j phibar_j^{n+1} - D1_j(k c^n).
-// These are the 2D kernels: a CTA of 32 x 16 threads on a 128 x 16 tile, a
-// float4 of x points per thread (3D: kernels_pml3d.cu).
+// 3D: kernels_pml3d.cu.  2D: PML_U and PML_B run on the TMA shot-loop tiles
+// (EXT_PML of tma2d_tile.cuh); this file holds PML_PHI and PML_A, on the frame of
+// points that need them.
+//
+// Away from the layer the scheme is the leapfrog, and with lambda^n = k c^n so
+// is its adjoint: lambda^{n-1} = 2 lambda^n - lambda^{n+1} + k (L^T lambda^n +
+// P^T r^n).  So points farther than the layer width plus R from every face
+// (pml_near) take the leapfrog's update, and only the others PML_A and PML_B, with
+// three fields for both: `cur` holds lambda^n everywhere (near points: ubar^{n+1}
+// before PML_A), `other` lambda^{n+1}, then lambda^{n-1} (near: ubar^n), and a
+// third the near points' share of ubar^{n-1}.  The phi adjoints are kept as
+// psi_j = b_j phibar_j, so that PML_A needs no b_j at its stencil's points.
 #include "fwi_internal.cuh"
 
 namespace fwi {
@@ -32,188 +42,111 @@ __device__ __forceinline__ float4 ldg4(const float* q) {
 }
 __device__ __forceinline__ float4 ld4(const float* q) { return *reinterpret_cast<const float4*>(q); }
 __device__ __forceinline__ void st4(float* q, const float4& v) { *reinterpret_cast<float4*>(q) = v; }
-__device__ __forceinline__ float4 mul4(const float4& a, const float4& b) {
-  return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
-}
 __device__ __forceinline__ void unpack(const float4& t, float* v) {
   v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
 __device__ __forceinline__ float4 pack(const float* v) { return make_float4(v[0], v[1], v[2], v[3]); }
 
-// A_j at index i of an axis of n points (0 outside the grid).
-__device__ __forceinline__ float sp_at(const float* sp, int i, int n) {
-  return (i >= 0 && i < n) ? sp[i] : 0.f;
-}
-// b_j of axis j from A_j and the other axes' A_k, A_l.
-__device__ __forceinline__ float pml_b(float Aj, float Ak, float Al) {
-  return 2.f * ((Ak + Al) - Aj) / (1.f + Aj);
-}
-__device__ __forceinline__ float pml_p(float Aj) { return (1.f - Aj) / (1.f + Aj); }
-
-
-template <int R>
-struct Pml2 {
-  static constexpr int TX = EXT_TX2, TY = EXT_TY2;
-  static constexpr int XH = (R <= 4) ? 4 : 8, NL = XH / 4;
-  static constexpr int SW = TX / 4 + 2 * NL, SH = TY + 2 * R, QW = TX / 4;
-  static constexpr size_t SMEM = ((size_t)SH * SW + TY * SW + SH * QW) * 16;
+// The frame of points within W of a face, as float4 groups: row strips of
+// 32 groups x 8 rows per CTA (top, bottom), then the groups at both ends of the
+// rows between, 256 per CTA in linear order.
+struct Frame {
+  int ngx, yt, yb, gl, gr;   // rows [0, yt) and [yb, ny) whole, groups [0, gl) and [gr, ngx) else
+  int bx, nrow, ncol;        // CTAs per strip of 8 rows, of the row strips, of the rest
+  __host__ __device__ Frame(int nx, int ny, int W) {
+    ngx = (nx + 3) / 4;
+    yt = W < ny ? W : ny;
+    yb = ny - W > yt ? ny - W : yt;
+    gl = (W + 3) / 4 < ngx ? (W + 3) / 4 : ngx;
+    gr = (nx - W) / 4 > gl ? (nx - W) / 4 : gl;
+    bx = (ngx + 31) / 32;
+    nrow = bx * ((yt + 7) / 8 + (ny - yb + 7) / 8);
+    ncol = ((yb - yt) * (gl + ngx - gr) + 255) / 256;
+  }
+  // group and row of thread t of CTA b; false: none
+  __device__ __forceinline__ bool at(int b, int t, int ny, int* g, int* y) const {
+    if (b < nrow) {
+      const int strip = b / bx, top = (yt + 7) / 8;
+      *g = (b - strip * bx) * 32 + (t & 31);
+      *y = (strip < top ? 8 * strip : yb + 8 * (strip - top)) + (t >> 5);
+      return *g < ngx && *y < (strip < top ? yt : ny);
+    }
+    const int i = (b - nrow) * 256 + t, n = gl + ngx - gr;
+    *y = yt + i / n;
+    *g = i % n;
+    if (*g >= gl) *g += gr - gl;
+    return *y < yb;
+  }
 };
 
-template <int R, bool VD, int MODE>
-__global__ void __launch_bounds__(EXT_TX2 / 4 * EXT_TY2, 2) k_pml2d(const StepParams p) {
-  using G = Pml2<R>;
-  constexpr int TX = G::TX, TY = G::TY, NL = G::NL, SW = G::SW, SH = G::SH, QW = G::QW;
-  constexpr int XH = G::XH;
-  constexpr int NT = TX / 4 * TY;
+// PML_PHI on the layer, or PML_A on the points within the stencil's reach of it.
+//
+// Bound by latency and L2: a thread has some 13 float4 loads in flight and little
+// else.  A frame of groups instead of the 128 x 16 tiles that touch it (1024 x
+// 1024, a 20-point layer, 6 shots: PML_PHI 20.5 -> 9.0 us, PML_A 36 -> 10 us; the
+// tiles hold three times the frame's points).  With U and B on the shot-loop tiles
+// a time step of the gradient takes 111 us where four passes over one-shot tiles
+// of the whole grid took 195.
+template <int R, int MODE>
+__global__ void __launch_bounds__(256, 4) k_pml2d(const StepParams p) {
+  constexpr int NL = (R <= 4) ? 1 : 2;
   constexpr int NV = 4 + 8 * NL;
-  constexpr bool FULL = MODE != PML_A;     // the stencil input tile with halo
-  constexpr bool CROSS = MODE == PML_U || MODE == PML_A || (MODE == PML_B && VD);
-  extern __shared__ __align__(16) float4 sm[];
-  float4* s_x = sm;                        // [SH][SW]
-  float4* s_r = sm + SH * SW;              // tile rows with x halo [TY][SW]
-  float4* s_c = s_r + TY * SW;             // tile columns with y halo [SH][QW]
-
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int tid = ty * (TX / 4) + tx;
-  const int b = blockIdx.z;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const long long fo = (long long)b * p.fstride;
-  if (MODE == PML_PHI) {   // phi changes only inside the layer
-    if (!(x0 < p.nb || x0 + TX > p.nx - p.nb || y0 < p.nb || y0 + TY > p.ny - p.nb)) return;
-  }
-  // phi (phibar) matter only in the layer and are read within R of it: tiles
-  // farther away skip them (phi is 0 there; phibar is never read there)
-  const int reach = p.nb + R;
-  const bool near = x0 < reach || x0 + TX > p.nx - reach || y0 < reach || y0 + TY > p.ny - reach;
-  if (MODE == PML_U) {
-    const long long blk = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    sample_receivers(p, blk * NT + tid);
-  }
-  const float* __restrict__ X = p.x + fo;
-  const long long base = (long long)(y0 + p.oy - R) * p.sx + (x0 + p.ox - XH);
-  if (FULL) {
-    for (int i = tid; i < SH * SW; i += NT) {
-      const int r = i / SW, c = i - r * SW;
-      const long long o = base + (long long)r * p.sx + 4 * c;
-      const float4 xv = ldg4(X + o);
-      s_x[i] = (MODE == PML_B) ? mul4(ldg4(p.kf + o), xv) : xv;
-    }
-  }
-  const bool cross = CROSS && (near || MODE == PML_B);
-  if (cross) {
-    for (int i = tid; i < TY * SW; i += NT) {
-      const int r = i / SW, c = i - r * SW;
-      const long long o = base + (long long)(r + R) * p.sx + 4 * c;
-      if (MODE == PML_U) {
-        s_r[i] = ldg4(p.ph[0] + fo + o);
-      } else if (MODE == PML_A) {     // b_x phibar_x
-        float f[4];
-        unpack(ldg4(p.ph[0] + fo + o), f);
-        const float Ay = sp_at(p.spy, y0 + r, p.ny);
-#pragma unroll
-        for (int l = 0; l < 4; ++l) f[l] *= pml_b(sp_at(p.spx, x0 - XH + 4 * c + l, p.nx), Ay, 0.f);
-        s_r[i] = pack(f);
-      } else {                        // b_x k c
-        s_r[i] = mul4(ldg4(p.bx + o), mul4(ldg4(p.kf + o), ldg4(X + o)));
-      }
-    }
-    for (int i = tid; i < SH * QW; i += NT) {
-      const int r = i / QW, c = i - r * QW;
-      const long long o = base + (long long)r * p.sx + 4 * (c + NL);
-      if (MODE == PML_U) {
-        s_c[i] = ldg4(p.ph[1] + fo + o);
-      } else if (MODE == PML_A) {     // b_y phibar_y
-        float f[4];
-        unpack(ldg4(p.ph[1] + fo + o), f);
-        const float Ay = sp_at(p.spy, y0 - R + r, p.ny);
-#pragma unroll
-        for (int l = 0; l < 4; ++l) f[l] *= pml_b(Ay, sp_at(p.spx, x0 + 4 * c + l, p.nx), 0.f);
-        s_c[i] = pack(f);
-      } else {                        // b_y k c
-        s_c[i] = mul4(ldg4(p.by + o), mul4(ldg4(p.kf + o), ldg4(X + o)));
-      }
-    }
-  }
-  __syncthreads();
-
-  const int ly = ty, yg = y0 + ly, srow = ly + R;
-  const int xg = x0 + 4 * tx;
-  const long long pi = (long long)(yg + p.oy) * p.sx + (xg + p.ox);
+  const Frame F(p.nx, p.ny, MODE == PML_PHI ? p.nb : p.nb + R);
+  int g, yg;
+  if (!F.at(blockIdx.x, threadIdx.x, p.ny, &g, &yg)) return;
+  const int b = blockIdx.y;
+  const int xg = 4 * g;
+  const int pix = (yg + p.oy) * p.sx + (xg + p.ox);
+  const long long pi = (long long)b * p.fstride + pix;
   bool in[4];
 #pragma unroll
-  for (int l = 0; l < 4; ++l) in[l] = (yg < p.ny) && (xg + l < p.nx);
+  for (int l = 0; l < 4; ++l) in[l] = xg + l < p.nx;
+
+  // D1x and D1y of u^{n+1}, or of psi_x = b_x phibar_x and psi_y = b_y phibar_y
+  const float* row = (MODE == PML_PHI ? p.x : p.ph[0]) + pi;
+  const float* col = (MODE == PML_PHI ? p.x : p.ph[1]) + pi;
+  float d1x[4] = {0.f, 0.f, 0.f, 0.f}, d1y[4] = {0.f, 0.f, 0.f, 0.f};
+  float v[NV];
+#pragma unroll
+  for (int q = 0; q <= 2 * NL; ++q) unpack(ld4(row + 4 * (q - NL)), v + 4 * q);
+#pragma unroll
+  for (int l = 0; l < 4; ++l)
+#pragma unroll
+    for (int j = 1; j <= R; ++j) d1x[l] = fmaf(p.wx.w1[j], v[4 * NL + l + j] - v[4 * NL + l - j], d1x[l]);
+#pragma unroll
+  for (int j = 1; j <= R; ++j) {
+    float a[4], c[4];
+    unpack(ld4(col - j * p.sx), a);
+    unpack(ld4(col + j * p.sx), c);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) d1y[l] = fmaf(p.wy.w1[j], c[l] - a[l], d1y[l]);
+  }
   float Ax[4];
   unpack(ldg4(p.spx + xg), Ax);
   const float Ay = p.spy[yg];
-
-  float v[NV], cen[4] = {0.f, 0.f, 0.f, 0.f}, acc[4] = {0.f, 0.f, 0.f, 0.f};
-  float d1x[4] = {0.f, 0.f, 0.f, 0.f}, d1y[4] = {0.f, 0.f, 0.f, 0.f};
-  if (FULL) {
-#pragma unroll
-    for (int q = 0; q <= 2 * NL; ++q) unpack(s_x[srow * SW + tx + q], v + 4 * q);
-    float c2[4];
+  if (MODE == PML_PHI) {
+    float fx[4], fy[4];
+    unpack(ld4(p.ph[0] + pi), fx);
+    unpack(ld4(p.ph[1] + pi), fy);
 #pragma unroll
     for (int l = 0; l < 4; ++l) {
-      const int c = 4 * NL + l;
-      cen[l] = v[c];
-      c2[l] = v[c] + v[c];
-      if (MODE != PML_PHI) {
-#pragma unroll
-        for (int j = 1; j <= R; ++j) acc[l] = fmaf(p.wx.w2[j], (v[c + j] + v[c - j]) - c2[l], acc[l]);
-      }
-#pragma unroll
-      for (int j = 1; j <= R; ++j) d1x[l] = fmaf(p.wx.w1[j], v[c + j] - v[c - j], d1x[l]);
+      fx[l] = in[l] ? ((1.f - Ax[l]) * fx[l] + 2.f * (Ay - Ax[l]) * d1x[l]) / (1.f + Ax[l]) : 0.f;
+      fy[l] = in[l] ? ((1.f - Ay) * fy[l] + 2.f * (Ax[l] - Ay) * d1y[l]) / (1.f + Ay) : 0.f;
     }
-#pragma unroll
-    for (int j = 1; j <= R; ++j) {
-      float a[4], cc[4];
-      unpack(s_x[(srow - j) * SW + tx + NL], a);
-      unpack(s_x[(srow + j) * SW + tx + NL], cc);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        if (MODE != PML_PHI) acc[l] = fmaf(p.wy.w2[j], (a[l] + cc[l]) - c2[l], acc[l]);
-        d1y[l] = fmaf(p.wy.w1[j], cc[l] - a[l], d1y[l]);
-      }
-    }
+    st4(p.ph[0] + pi, pack(fx));
+    st4(p.ph[1] + pi, pack(fy));
+    return;
   }
-  if (MODE == PML_U && VD) {   // L_rho u = lap u - b . grad u
-    float bxv[4], byv[4];
-    unpack(ldg4(p.bx + pi), bxv);
-    unpack(ldg4(p.by + pi), byv);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) acc[l] -= bxv[l] * d1x[l] + byv[l] * d1y[l];
-  }
-  // D1x of the row tile and D1y of the column tile: phi (PML_U), b phibar
-  // (PML_A), b k c (PML_B, variable density)
-  float dr[4] = {0.f, 0.f, 0.f, 0.f};
-  if (cross) {
-    float w[NV];
-#pragma unroll
-    for (int q = 0; q <= 2 * NL; ++q) unpack(s_r[ly * SW + tx + q], w + 4 * q);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const int c = 4 * NL + l;
-#pragma unroll
-      for (int j = 1; j <= R; ++j) dr[l] = fmaf(p.wx.w1[j], w[c + j] - w[c - j], dr[l]);
-    }
-#pragma unroll
-    for (int j = 1; j <= R; ++j) {
-      float a[4], cc[4];
-      unpack(s_c[(srow - j) * QW + tx], a);
-      unpack(s_c[(srow + j) * QW + tx], cc);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) dr[l] = fmaf(p.wy.w1[j], cc[l] - a[l], dr[l]);
-    }
-  }
-  // sources (PML_U) or the residual of step n-1 (PML_A): this row's entries
+  // PML_A: the residual of step n-1 (this row's entries)
   float inj[4] = {0.f, 0.f, 0.f, 0.f};
-  if ((MODE == PML_U || MODE == PML_A) && p.inj_off) {
-    const int t = b * p.ntiles + blockIdx.y * gridDim.x + blockIdx.x;
+  if (p.inj_off) {
+    const int t = b * p.ntiles + (yg / EXT_TY2) * ((p.nx + EXT_TX2 - 1) / EXT_TX2) + xg / EXT_TX2;
     if (p.inj_off[t + 1] > p.inj_off[t]) {
-      const int* rr = p.inj_row + (size_t)t * (TY + 1);
-      const int r1 = rr[ly + 1];
-      for (int e = rr[ly]; e < r1; ++e) {
-        const int elx = p.inj_loc[e] - ly * TX;
+      const int ly = yg % EXT_TY2, tx = (xg % EXT_TX2) / 4;
+      const int* rr = p.inj_row + (size_t)t * (EXT_TY2 + 1) + ly;
+      const int r1 = rr[1];
+      for (int e = rr[0]; e < r1; ++e) {
+        const int elx = p.inj_loc[e] - ly * EXT_TX2;
         if ((elx >> 2) == tx) {
           const float val = p.inj_w[e] * p.vals[p.inj_vidx[e] + p.step_off];
           const int l = elx & 3;
@@ -223,112 +156,46 @@ __global__ void __launch_bounds__(EXT_TX2 / 4 * EXT_TY2, 2) k_pml2d(const StepPa
       }
     }
   }
-
-  if (MODE == PML_U) {
-    float k[4], uo[4], r[4], h[4];
-    unpack(ldg4(p.kf + pi), k);
-    unpack(ld4(p.up + fo + pi), uo);
+  float k[4], xn[4], xc[4], un[4], lam[4];
+  unpack(ldg4(p.kf + pix), k);
+  unpack(ld4(p.up + pi), xn);
+  unpack(ld4(p.hist2 + pi), xc);
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const float E = (acc[l] + inj[l]) + dr[l];
-      const float a = Ax[l] + Ay;
-      const float e = 4.f * Ax[l] * Ay;
-      const float hv = k[l] * E;
-      const float rv = (2.f * cen[l] - (1.f - a) * uo[l] - e * cen[l] + hv) / (1.f + a);
-      r[l] = in[l] ? rv : 0.f;
-      h[l] = in[l] ? hv : 0.f;
-    }
-    st4(p.up + fo + pi, pack(r));
-    if (p.hist) __stcs(reinterpret_cast<float4*>(p.hist + fo + pi), pack(h));
-  } else if (MODE == PML_PHI) {
-    float fx[4], fy[4];
-    unpack(ld4(p.ph[0] + fo + pi), fx);
-    unpack(ld4(p.ph[1] + fo + pi), fy);
+  for (int l = 0; l < 4; ++l) {
+    const float a = Ax[l] + Ay, e = 4.f * Ax[l] * Ay;
+    const float c = (xn[l] - (d1x[l] + d1y[l])) / (1.f + a);
+    lam[l] = in[l] ? k[l] * c : 0.f;
+    un[l] = in[l] ? inj[l] - (1.f - a) * c : 0.f;
+    xc[l] = in[l] ? xc[l] + (2.f - e) * c : 0.f;
+  }
+  st4(p.up + pi, pack(lam));
+  st4(p.hist2 + pi, pack(un));
+  st4(p.out + pi, pack(xc));
+  if (p.image) {
+    float h[4], gr[4];
+    unpack(__ldcs(reinterpret_cast<const float4*>(p.hist + pi)), h);
+    unpack(ld4(p.g + pi), gr);
 #pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const float nx_ = pml_p(Ax[l]) * fx[l] + pml_b(Ax[l], Ay, 0.f) * d1x[l];
-      const float ny_ = pml_p(Ay) * fy[l] + pml_b(Ay, Ax[l], 0.f) * d1y[l];
-      fx[l] = in[l] ? nx_ : 0.f;
-      fy[l] = in[l] ? ny_ : 0.f;
-    }
-    st4(p.ph[0] + fo + pi, pack(fx));
-    st4(p.ph[1] + fo + pi, pack(fy));
-  } else if (MODE == PML_A) {
-    float k[4], xn[4], h[4], g[4], cc[4], un[4];
-    unpack(ldg4(p.kf + pi), k);
-    unpack(ld4(p.up + fo + pi), xn);
-    unpack(__ldcs(reinterpret_cast<const float4*>(p.hist + fo + pi)), h);
-    unpack(ld4(p.g + fo + pi), g);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const float a = Ax[l] + Ay;
-      const float c = (xn[l] - dr[l]) / (1.f + a);
-      cc[l] = in[l] ? c : 0.f;
-      un[l] = in[l] ? inj[l] - (1.f - a) * c : 0.f;
-      if (in[l]) g[l] = fmaf(-(k[l] * c), h[l], g[l]);
-    }
-    st4(p.out + fo + pi, pack(cc));
-    st4(p.up + fo + pi, pack(un));
-    st4(p.g + fo + pi, pack(g));
-  } else {   // PML_B
-    float c[4], xc[4];
-    unpack(ld4(p.x + fo + pi), c);
-    unpack(ld4(p.up + fo + pi), xc);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const float e = 4.f * Ax[l] * Ay;
-      const float LT = acc[l] + (VD ? dr[l] : 0.f);
-      const float nxc = xc[l] + ((2.f - e) * c[l] + LT);
-      xc[l] = in[l] ? nxc : 0.f;
-    }
-    st4(p.up + fo + pi, pack(xc));
-    if (near) {
-      float fx[4], fy[4];
-      unpack(ld4(p.ph[0] + fo + pi), fx);
-      unpack(ld4(p.ph[1] + fo + pi), fy);
-#pragma unroll
-      for (int l = 0; l < 4; ++l) {
-        const float nfx = pml_p(Ax[l]) * fx[l] - d1x[l];
-        const float nfy = pml_p(Ay) * fy[l] - d1y[l];
-        fx[l] = in[l] ? nfx : 0.f;
-        fy[l] = in[l] ? nfy : 0.f;
-      }
-      st4(p.ph[0] + fo + pi, pack(fx));
-      st4(p.ph[1] + fo + pi, pack(fy));
-    }
+    for (int l = 0; l < 4; ++l)
+      if (in[l]) gr[l] = fmaf(-lam[l], h[l], gr[l]);
+    st4(p.g + pi, pack(gr));
   }
 }
 
-template <int R, bool VD, int MODE>
+template <int R, int MODE>
 cudaError_t launch_m(const StepParams& p, cudaStream_t st) {
-  constexpr size_t smem = Pml2<R>::SMEM;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_pml2d<R, VD, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  dim3 grid((p.nx + EXT_TX2 - 1) / EXT_TX2, (p.ny + EXT_TY2 - 1) / EXT_TY2, p.B);
-  k_pml2d<R, VD, MODE><<<grid, dim3(EXT_TX2 / 4, EXT_TY2), smem, st>>>(p);
+  const Frame F(p.nx, p.ny, MODE == PML_PHI ? p.nb : p.nb + R);
+  if (F.nrow + F.ncol == 0) return cudaSuccess;   // (no layer)
+  k_pml2d<R, MODE><<<dim3(F.nrow + F.ncol, p.B), 256, 0, st>>>(p);
   return cudaGetLastError();
-}
-
-template <int R, bool VD>
-cudaError_t launch_mode(const StepParams& p, int mode, cudaStream_t st) {
-  switch (mode) {
-    case PML_U: return launch_m<R, VD, PML_U>(p, st);
-    case PML_PHI: return launch_m<R, VD, PML_PHI>(p, st);
-    case PML_A: return launch_m<R, VD, PML_A>(p, st);
-    default: return launch_m<R, VD, PML_B>(p, st);
-  }
 }
 
 }  // namespace
 
-cudaError_t launch_pml2d(const StepParams& p, int R, bool vd, int mode, cudaStream_t st) {
-  if (R == 4) return vd ? launch_mode<4, true>(p, mode, st) : launch_mode<4, false>(p, mode, st);
-  return vd ? launch_mode<5, true>(p, mode, st) : launch_mode<5, false>(p, mode, st);
+cudaError_t launch_pml2d(const StepParams& p, int R, int mode, cudaStream_t st) {
+  if (mode == PML_PHI) return R == 4 ? launch_m<4, PML_PHI>(p, st) : launch_m<5, PML_PHI>(p, st);
+  if (mode == PML_A) return R == 4 ? launch_m<4, PML_A>(p, st) : launch_m<5, PML_A>(p, st);
+  return cudaErrorInvalidValue;   // (PML_U and PML_B: EXT_PML of kernels2d_tma_ext.cu)
 }
 
 }  // namespace fwi
@@ -341,7 +208,7 @@ namespace {
 // thread per bucket in its entries' order (no two tiles share a node): the
 // receiver residuals of one step spread onto an adjoint field.
 __global__ void k_inject_buckets(const StepParams p, float* __restrict__ field, int tx, int ty,
-                                 int zc, int gx, int gy, int nbuckets) {
+                                 int zc, int gx, int gy, int reach, int nbuckets) {
   const int bk = blockIdx.x * blockDim.x + threadIdx.x;
   if (bk >= nbuckets) return;
   const int slot = bk / p.ntiles, t = bk - slot * p.ntiles;
@@ -350,6 +217,7 @@ __global__ void k_inject_buckets(const StepParams p, float* __restrict__ field, 
   for (int e = p.inj_off[bk]; e < p.inj_off[bk + 1]; ++e) {
     const int loc = p.inj_loc[e];
     const int lx = loc % tx, ly = (loc / tx) % ty, lz = loc / (tx * ty);
+    if (reach > 0 && !pml_near((bx * tx + lx) & ~3, by * ty + ly, reach, p.nx, p.ny)) continue;
     const long long idx = (long long)(bz * zc + lz + p.oz) * p.sxy +
                           (long long)(by * ty + ly + p.oy) * p.sx + (bx * tx + lx + p.ox);
     f[idx] += p.inj_w[e] * p.vals[p.inj_vidx[e] + p.step_off];
@@ -359,10 +227,10 @@ __global__ void k_inject_buckets(const StepParams p, float* __restrict__ field, 
 }  // namespace
 
 cudaError_t launch_inject_buckets(const StepParams& p, float* field, int tx, int ty, int zc, int gx,
-                                  int gy, cudaStream_t st) {
+                                  int gy, int reach, cudaStream_t st) {
   const int n = p.B * p.ntiles;
   if (n <= 0 || !p.inj_off) return cudaSuccess;
-  k_inject_buckets<<<(n + 127) / 128, 128, 0, st>>>(p, field, tx, ty, zc, gx, gy, n);
+  k_inject_buckets<<<(n + 127) / 128, 128, 0, st>>>(p, field, tx, ty, zc, gx, gy, reach, n);
   return cudaGetLastError();
 }
 

@@ -418,13 +418,11 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
     return fail(FWI_ERR_INVALID_ARG, "tile variant out of range");
   out.sc = sc;
   if (sc.ext()) {
-    // the extended schemes have one tile shape: in 2D (sponge boundary) the
-    // TMA shot-loop kernels of 128 x 16 tiles (variant 6), otherwise one
-    // shot per CTA (kernels_ext.cu, kernels_pml.cu)
-    // in 3D the two-point plane-ring kernels take the fourth-order scheme and
-    // the attenuation (variant 12; y = 2 where its two fields fit); the PML
-    // keeps kernels_pml.cu
-    const bool tma2 = P->grid.ndim == 2 && !sc.pml;
+    // the extended schemes have one tile shape: in 2D the TMA shot-loop
+    // kernels of 128 x 16 tiles (variant 6)
+    // in 3D the two-point plane-ring kernels (variant 12; y = 2 where its two
+    // fields fit)
+    const bool tma2 = P->grid.ndim == 2;
     const bool x2 = P->grid.ndim == 3 && (sc.pml || sc.t4 || sc.att == 0 || sc.ring);
     out.tile = tma2 ? 6 : (x2 ? 12 : 0);
     out.shape = tma2 ? 1 : (x2 ? 3 : 0);

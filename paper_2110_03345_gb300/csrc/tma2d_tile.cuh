@@ -143,8 +143,8 @@ __device__ __forceinline__ void prefetch_l2(const void* q) {
 // samp_rank is the CTA's rank among its problem's CTAs, gx the problem's tile
 // count along x.
 // MODE selects the update: LEAP the leapfrog of this file's header, or one
-// of the extended schemes (EXT_KW, EXT_T4, EXT_ATT0, EXT_ATT2 of
-// fwi_internal.cuh, the arithmetic of kernels_ext.cu) on the same pipeline:
+// of the extended schemes (EXT_KW, EXT_T4, EXT_ATT0, EXT_ATT2, EXT_PML of
+// fwi_internal.cuh) on the same pipeline:
 // the stencil input x is the TMA tile (u, lambda, or the k w / k L^T lambda
 // scratch of the fourth-order scheme), the model data of the tile (k, the
 // attenuation coefficient, its tiles for the y = 2 adjoint) are loaded once
@@ -215,6 +215,10 @@ __device__ __forceinline__ void step2d_tma_tile(const StepParams& p, const AxisW
   const int xg = x0 + 4 * tx;
   const int base = (y0 + p.oy - R) * p.sx + (x0 + p.ox - G::XH);
   const float4 ax4 = ldg4(p.spx + xg);
+  // PML: this thread's points come within the stencil's reach of the layer
+  constexpr bool PM = MODE == EXT_PML;
+  static_assert(!PM || RY == 1, "");
+  const bool near = PM && pml_near(xg, y0 + ty, p.nb + R, p.nx, p.ny);
   int pix[RY];
   float4 kk[RY];
   float4 atv[AT ? RY : 1];
@@ -318,6 +322,32 @@ __device__ __forceinline__ void step2d_tma_tile(const StepParams& p, const AxisW
       if (VD && !ADJ) {
         bxf[iy] = ldg4(p.bx + pix[iy]);
         byf[iy] = ldg4(p.by + pix[iy]);
+      }
+    }
+    // PML: D1x phi_x + D1y phi_y of the points near the layer, before the wait
+    float dr[PM && !ADJ ? 4 : 1];
+    if constexpr (PM && !ADJ) {
+#pragma unroll
+      for (int ix = 0; ix < 4; ++ix) dr[ix] = 0.f;
+      if (near) {
+        const float* const fx = p.ph[0] + (size_t)s * p.fstride + pix[0];
+        const float* const fy = p.ph[1] + (size_t)s * p.fstride + pix[0];
+        float w[NV];
+#pragma unroll
+        for (int q = 0; q <= 2 * NL; ++q) unpack(ld4(fx + 4 * (q - NL)), w + 4 * q);
+#pragma unroll
+        for (int ix = 0; ix < 4; ++ix)
+#pragma unroll
+          for (int j = 1; j <= R; ++j)
+            dr[ix] = fmaf(wx.w1[j], w[4 * NL + ix + j] - w[4 * NL + ix - j], dr[ix]);
+#pragma unroll
+        for (int j = 1; j <= R; ++j) {
+          float a[4], c[4];
+          unpack(ld4(fy - j * p.sx), a);
+          unpack(ld4(fy + j * p.sx), c);
+#pragma unroll
+          for (int ix = 0; ix < 4; ++ix) dr[ix] = fmaf(wy.w1[j], c[ix] - a[ix], dr[ix]);
+        }
       }
     }
     // A wait that times out flags the error and carries on (no early exit, so
@@ -463,7 +493,7 @@ __device__ __forceinline__ void step2d_tma_tile(const StepParams& p, const AxisW
                           lc[ix]);
         }
       }
-      if (e1 > e0) {
+      if (e1 > e0 && !(PM && ADJ && near)) {
         // only this row's entries (the bucket's per-row ranges)
         const int* rr = p.inj_row + (size_t)(s * p.ntiles + tile_id) * (TY + 1);
         int e = rr[ly], r1 = rr[ly + 1];
@@ -491,13 +521,89 @@ __device__ __forceinline__ void step2d_tma_tile(const StepParams& p, const AxisW
         for (; e < r1; ++e) {
           const int elx = p.inj_loc[e] - ly * TX;
           if ((elx >> 2) == tx) {
-            const float w = (MODE == LEAP) ? p.inj_w[e] : p.inj_scale * p.inj_w[e];
+            const float w = (MODE == LEAP || PM) ? p.inj_w[e] : p.inj_scale * p.inj_w[e];
             const float val = w * p.vals[p.inj_vidx[e] + p.step_off];
             const int ix = elx & 3;
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[q] += (q == ix) ? val : 0.f;
           }
         }
+      }
+      if constexpr (PM) {
+        const size_t o = (size_t)s * p.fstride + pix[iy];
+        const float4 uo4 = s_uo[buf * TY * QW + ly * QW + tx];
+        float r[4], h[4];
+        if (near && ADJ) {    // ubar^n += L^T lambda^n; psi_j = p_j psi_j - b_j D1_j lambda^n
+#pragma unroll
+          for (int ix = 0; ix < 4; ++ix)
+            r[ix] = (yg < p.ny && xg + ix < p.nx) ? get(uo4, ix) + acc[ix] : 0.f;
+          st4(up_s + pix[iy], make_float4(r[0], r[1], r[2], r[3]));
+          if (pml_near(xg, yg, p.nb, p.nx, p.ny)) {
+            float* const fx = p.ph[0] + o;
+            float* const fy = p.ph[1] + o;
+            float f[4], d[4];
+            // (the window is read again: held here it would spill)
+            asm volatile("" ::: "memory");
+#pragma unroll
+            for (int q = 0; q <= 2 * NL; ++q) unpack(s_u[srow * SW + tx + q], v + 4 * q);
+            unpack(ld4(fx), f);
+#pragma unroll
+            for (int ix = 0; ix < 4; ++ix) {
+              const float A = get(ax4, ix);
+              const int c = 4 * NL + ix;
+              d[ix] = 0.f;
+#pragma unroll
+              for (int j = 1; j <= R; ++j) d[ix] = fmaf(wx.w1[j], v[c + j] - v[c - j], d[ix]);
+              f[ix] = ((1.f - A) * f[ix] - 2.f * (ay[iy] - A) * d[ix]) / (1.f + A);
+              if (yg >= p.ny || xg + ix >= p.nx) f[ix] = 0.f;
+              d[ix] = 0.f;
+            }
+            st4(fx, make_float4(f[0], f[1], f[2], f[3]));
+            asm volatile("" ::: "memory");
+#pragma unroll
+            for (int j = 1; j <= R; ++j) {
+              float a[4], c[4];
+              unpack(s_u[(srow - j) * SW + tx + NL], a);
+              unpack(s_u[(srow + j) * SW + tx + NL], c);
+#pragma unroll
+              for (int ix = 0; ix < 4; ++ix) d[ix] = fmaf(wy.w1[j], c[ix] - a[ix], d[ix]);
+            }
+            unpack(ld4(fy), f);
+#pragma unroll
+            for (int ix = 0; ix < 4; ++ix) {
+              f[ix] = ((1.f - ay[iy]) * f[ix] - 2.f * (get(ax4, ix) - ay[iy]) * d[ix]) / (1.f + ay[iy]);
+              if (yg >= p.ny || xg + ix >= p.nx) f[ix] = 0.f;
+            }
+            st4(fy, make_float4(f[0], f[1], f[2], f[3]));
+          }
+          continue;
+        }
+#pragma unroll
+        for (int ix = 0; ix < 4; ++ix) {
+          const float cen = v[4 * NL + ix];
+          h[ix] = get(kk[iy], ix) * (ADJ ? acc[ix] : acc[ix] + dr[ADJ ? 0 : ix]);
+          if (!ADJ && near) {
+            const float ax = get(ax4, ix), a = ax + ay[iy], e = 4.f * ax * ay[iy];
+            r[ix] = (2.f * cen - (1.f - a) * get(uo4, ix) - e * cen + h[ix]) / (1.f + a);
+          } else {
+            r[ix] = (2.f * cen - get(uo4, ix)) + h[ix];
+          }
+        }
+#pragma unroll
+        for (int ix = 0; ix < 4; ++ix) {
+          const bool in = (yg < p.ny) && (xg + ix < p.nx);
+          r[ix] = in ? r[ix] : 0.f;
+          if (!ADJ) h[ix] = in ? h[ix] : 0.f;
+        }
+        st4(up_s + pix[iy], make_float4(r[0], r[1], r[2], r[3]));
+        if (!ADJ) {
+          if (h_s) __stcs(reinterpret_cast<float4*>(h_s + pix[iy]), make_float4(h[0], h[1], h[2], h[3]));
+        } else if (p.image) {
+          const float4 hv4 = s_hv[buf * TY * QW + ly * QW + tx];
+#pragma unroll
+          for (int ix = 0; ix < 4; ++ix) gs[iy][ix] = fmaf(v[4 * NL + ix], get(hv4, ix), gs[iy][ix]);
+        }
+        continue;
       }
       if (MODE != LEAP) {
         const int so = buf * TY * QW + ly * QW + tx;   // this thread's float4 in a staged tile
@@ -549,7 +655,7 @@ __device__ __forceinline__ void step2d_tma_tile(const StepParams& p, const AxisW
       issue(k + 2);
     }
   }
-  if (ADJ && MODE != EXT_KW && p.image) {
+  if (ADJ && MODE != EXT_KW && p.image && !near) {
     // g_group -= sum over this group's shots of lambda^k h^k
     float* gbase = p.g + (size_t)grp * p.fstride;
 #pragma unroll
