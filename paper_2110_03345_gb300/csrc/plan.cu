@@ -340,14 +340,36 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc) {
   return FWI_OK;
 }
 
-// Shots per CTA of the 2D per-step kernels for B shots: six share a tile's
-// model loads and gradient update; at least four waves of CTAs (two resident
-// per SM) keep the SMs balanced.
-int shot_group(const fwi_plan* P, int shape, int B) {
-  const int T = tile_geo(P, shape, true).ntiles();
-  int S = std::min(B, 6);
-  while (S > 1 && (long long)T * ((B + S - 1) / S) < 8LL * P->nsm) --S;
-  return S;
+// Shots per CTA (S) of a 2D per-step launch over problems of (tiles, shots).  In
+// shot times, a CTA of S shots takes about S + 1 (the model loads and the gradient
+// update cost one), two CTAs per SM work at a time, and `tail` of a CTA is waited
+// for at the end of the step: about half, more in the extended schemes, whose CTAs
+// differ (the PML's 1024 x 1024 gradient of 6 shots: S = 3 27.3 ms, S = 6 29.0 ms).
+// The S with the least of the sum is taken.
+// Measured against the largest S <= 6 that leaves four waves of CTAs, us per
+// gradient step pair (8th order, density): 456 x 485, 16 shots 50.8 -> 39.8; 700 x
+// 748, 6 shots 43.3 -> 32.8, 10 shots 70.0 -> 47.9; 1024 x 1024, 6 shots 62.9 ->
+// 56.7, 8 shots 80.0 -> 74.9, 15 shots 132.9 -> 128.6; 1600 x 1600, 16 shots 333.9 ->
+// 311.4; 6 shots of the fourth-order scheme (800 x 872) 80.6 -> 76.1, of the PML
+// (1024 x 1024) 106.8 -> 103.9.
+int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail) {
+  int most = 1, best = 1;
+  for (const auto& ts : tiles_shots) most = std::max(most, ts.second);
+  double least = 0.0;
+  for (int S = 1; S <= most; ++S) {
+    double c = tail * (S + 1);
+    for (const auto& ts : tiles_shots)
+      c += (double)ts.first * (ts.second + (ts.second + S - 1) / S) / (2.0 * nsm);
+    if (S == 1 || c < least) {
+      least = c;
+      best = S;
+    }
+  }
+  return best;
+}
+
+int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc) {
+  return shot_group(P->nsm, {{tile_geo(P, shape, true).ntiles(), B}}, sc.ext() ? 0.75 : GROUP_TAIL);
 }
 
 // Planes per CTA of the default 3D variant.  A CTA spends about zc + 4 plane
@@ -450,7 +472,7 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
   if (out.res.on) {
     // (each shot has its own gradient slot)
   } else if (out.tma && P->grid.ndim == 2) {   // the 3D kernels take one shot per CTA
-    out.S = P->opt.shots_per_cta > 0 ? std::min(P->opt.shots_per_cta, B) : shot_group(P, out.shape, B);
+    out.S = P->opt.shots_per_cta > 0 ? std::min(P->opt.shots_per_cta, B) : shot_group(P, out.shape, B, sc);
   }
   out.bytes = fixed_bytes(P, g, vd, B, sc) + res_bytes + (size_t)B * slot_bytes(P, g, grad, K, sc);
   if (split)

@@ -36,22 +36,25 @@ int most_entries(const fwi_plan* P, const double* xyz, long long n, int TH, int 
 
 }  // namespace
 
-// Whether a call of B shots may run resident.  Resident launches win while the per-step kernels find too few CTAs to share
-// a tile among shots: measured on a GB300 in us per step (per step pair for
-// gradients), per-step -> resident, 8th order with density: 256 x 256, one shot
-// 4.1 -> 2.3 forward and 9.1 -> 4.6 gradient; 700 x 748, one shot 4.5 -> 3.2 and
-// 11.0 -> 8.0; 1024 x 1024, one shot 6.4 -> 4.4 and 17.2 -> 9.7, four 17.6 -> 14.7
-// and 52.8 -> 35.5.  Forward runs break even where the per-step kernels group
-// two shots (1024 x 1024, six shots 21.5 -> 21.6; 456 x 485, 32 shots 23.1 ->
-// 30.0), gradients where they group three (1024 x 1024, eight shots 78.6 ->
-// 69.9, 16 shots 136.3 -> 138.8; 456 x 485, 32 shots 68.4 -> 77.8).
+// Whether a call of B shots may run resident.  A resident shot costs the same
+// whatever the number of shots; the per-step kernels' cost per shot falls as CTAs
+// of several shots fill the SMs.  Measured on a GB300 in us per step (per step pair
+// for gradients), per-step -> resident, 8th order with density: 256 x 256, one shot
+// 4.1 -> 2.3 forward and 9.1 -> 4.6 gradient; 700 x 748, two shots 5.9 -> 4.2 and
+// 14.7 -> 10.2; 1024 x 1024, one shot 5.9 -> 4.4 and 16.6 -> 10.5.  Forward runs
+// break even at about 8 tile-shots (128 x 16 points) per SM (456 x 485, twelve
+// shots 9.2 -> 9.3; 700 x 748, four 8.9 -> 7.9, six 11.7 -> 11.8; 1024 x 1024, two
+// 8.6 -> 8.2, three 11.3 -> 11.9), gradients at about 12.5 (456 x 485, 16 shots 29.1 ->
+// 28.5, twenty 32.6 -> 35.4; 700 x 748, six 31.3 -> 29.7, eight 38.5 -> 39.5; 1024 x
+// 1024, three 30.7 -> 29.9, four 38.2 -> 39.1).
 bool res_eligible(const fwi_plan* P, bool grad, int B, const Scheme& sc) {
   if (P->grid.ndim != 2 || sc.ext() || P->fixed_memory || P->per_step || P->opt.tile != 0 ||
       P->opt.shots_per_cta != 0 || B < 1 || P->nt < 2)
     return false;
   int id = 0, shape = 0;
   bool tma = false;
-  return resolve_tile(P, 0, &id, &shape, &tma) && shot_group(P, shape, B) <= (grad ? 2 : 1);
+  return resolve_tile(P, 0, &id, &shape, &tma) &&
+         2LL * tile_geo(P, shape, true).ntiles() * B <= (grad ? 25LL : 16LL) * P->nsm;
 }
 
 namespace {
