@@ -102,6 +102,7 @@ struct StepParams {
   float* ph[3];
   float dt;
   int nb;
+  const unsigned char* bflag;   // 3D plane rings: density gradients per plane and column (or null)
 };
 
 // Lanes per receiver sample: the 64- / 512-node sinc points split their
@@ -378,6 +379,12 @@ cudaError_t launch_res_combine(const float* raw, int nraw, int nslots, int steps
 cudaError_t launch_model_prep(const Layout& L, const float* vp, const float* rho, double dt,
                               int param, float* kf, float* lnr, unsigned int* stats,
                               cudaStream_t st);
+// flags[(z * gy + iy) * gx + ix], of the 64 x rows column tiles (gx x gy) and planes:
+// non-zero where the density terms (the adjoint's: b_x within R along x, b_y along y, b_z
+// along z) reach a non-zero b from the tile; count += the flags set
+cudaError_t launch_density_flags(const Layout& L, const float* bx, const float* by, const float* bz,
+                                 int rows, int gx, int gy, unsigned char* flags, unsigned int* count,
+                                 cudaStream_t st);
 cudaError_t launch_density_grad(const Layout& L, const float* lnr, const AxisW& wx,
                                 const AxisW& wy, const AxisW& wz, float* bx, float* by,
                                 float* bz, cudaStream_t st);

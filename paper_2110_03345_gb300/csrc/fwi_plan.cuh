@@ -68,6 +68,7 @@ struct fwi_plan {
   float* spx = nullptr;
   float* spy = nullptr;
   float* spz = nullptr;
+  unsigned char* bflag = nullptr;   // 3D: planes and columns with density gradients
   unsigned int* d_stats = nullptr;
   int* d_flags = nullptr;
   double* d_J = nullptr;     // per-batch misfit
@@ -250,6 +251,7 @@ struct Call {
   std::vector<MapEnt> maps;   // TMA descriptors of the wavefield buffers
   CUtensorMap hmap{};         // 2D TMA adjoint: the current batch's history buffer
   CUtensorMap h2map{};        // and its second history field (fourth-order scheme)
+  bool few_b = false;   // 3D: density terms only on the planes that P->bflag marks
   bool hmap_ok = false, h2map_ok = false;
   std::vector<float*> fstate; // forward state besides u^n, u^{n-1} (checkpointed with them)
   int64_t launches = 0;

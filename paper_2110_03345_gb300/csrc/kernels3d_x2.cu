@@ -27,23 +27,23 @@ namespace fwi {
 
 namespace {
 
-template <int R, bool VD, bool ADJ, int BY, bool CROWD = false>
+template <int R, bool VD, bool ADJ, int BY, bool CROWD = false, bool PP = false>
 cudaError_t launch_t(const StepParams& p, const CUtensorMap& um, const CUtensorMap& bxm,
                      const CUtensorMap& bym, const CUtensorMap* const* om, cudaStream_t st) {
   constexpr size_t smem = smem_bytes_x2<R, VD, ADJ, BY>();
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD>,
+    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD>,
+    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>,
                              cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   dim3 grid((p.nx + 63) / 64, (p.ny + BY - 1) / BY, p.B * p.nzc);
-  return launch_pdl(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD>, grid, dim3(32, BY), smem, st, p,
+  return launch_pdl(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>, grid, dim3(32, BY), smem, st, p,
                     um, bxm, bym, *om[0], *om[1], *om[2], *om[3]);
 }
 
@@ -51,7 +51,12 @@ template <int R, bool VD, bool ADJ>
 cudaError_t launch_tile(const StepParams& p, const CUtensorMap& um, const CUtensorMap& bxm,
                         const CUtensorMap& bym, const CUtensorMap* const* om, int tile,
                         cudaStream_t st) {
-  // (the 64 x 8 columns of the default variant have a crowded-plane instantiation)
+  // (the 64 x 8 columns of the default variant have a crowded-plane instantiation and
+  // one for models with few density gradients)
+  if constexpr (VD) {
+    if (tile3_variant(tile).by == 8 && !p.inj_crowded && p.bflag)
+      return launch_t<R, VD, ADJ, 8, false, true>(p, um, bxm, bym, om, st);
+  }
   if (tile3_variant(tile).by == 8)
     return p.inj_crowded ? launch_t<R, VD, ADJ, 8, true>(p, um, bxm, bym, om, st)
                          : launch_t<R, VD, ADJ, 8>(p, um, bxm, bym, om, st);

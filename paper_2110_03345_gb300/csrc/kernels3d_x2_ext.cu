@@ -17,22 +17,22 @@ namespace {
 
 constexpr int EXT3_BY = 8;
 
-template <int R, bool VD, bool ADJ, int MODE>
+template <int R, bool VD, bool ADJ, int MODE, bool PP = false>
 cudaError_t launch_e3(const StepParams& p, const CUtensorMap* const* m, cudaStream_t st) {
   constexpr size_t smem = smem_bytes_x2<R, VD, ADJ, EXT3_BY, MODE>();
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE>,
+    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE>,
+    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>,
                              cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   dim3 grid((p.nx + 63) / 64, (p.ny + EXT3_BY - 1) / EXT3_BY, p.B * p.nzc);
-  return launch_pdl(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE>, grid, dim3(32, EXT3_BY), smem, st, p,
+  return launch_pdl(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>, grid, dim3(32, EXT3_BY), smem, st, p,
                     *m[0], *m[1], *m[2], *m[3], *m[4], *m[5], *m[6]);
 }
 
@@ -42,7 +42,9 @@ cudaError_t launch_mode3(const StepParams& p, const CUtensorMap* const* m, int m
   switch (mode) {
     case EXT_KW: return launch_e3<R, VD, ADJ, EXT_KW>(p, m, st);
     case EXT_T4: return launch_e3<R, VD, ADJ, EXT_T4>(p, m, st);
-    case EXT_ATT2: return launch_e3<R, VD, ADJ, EXT_ATT2>(p, m, st);
+    case EXT_ATT2:
+      if (VD && p.bflag) return launch_e3<R, VD, ADJ, EXT_ATT2, VD>(p, m, st);
+      return launch_e3<R, VD, ADJ, EXT_ATT2>(p, m, st);
     default: return launch_e3<R, VD, ADJ, EXT_ATT0>(p, m, st);
   }
 }

@@ -112,8 +112,10 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
     pdl_wait();
     return;   // phi changes only inside the layer
   }
+  const unsigned long long bon = VD && (MODE == PML_U || MODE == PML_B) ? density_planes(p, z0, nz_c) : 0ull;
+  auto b_on = [&](int z) { return ((bon >> (z - z0)) & 1) != 0; };   // plane z has density gradients
   // planes whose row / column tiles matter
-  auto staged = [&](int z) { return MODE == PML_B || nearxy || nearz(z); };
+  auto staged = [&](int z) { return MODE == PML_B ? b_on(z) : (nearxy || nearz(z)); };
 
   const int tmx = x0 + p.ox - G::XOFF, tmy = y0 + p.oy - R, pz0 = z0 - R + p.oz;
   if (tid == 0) {
@@ -175,7 +177,7 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
   auto qc_val = [&](int lp, const float2& u) {
     const int z = z0 - R + lp;
     const long long id = (long long)(pz0 + lp) * p.sxy + col;
-    if (MODE == PML_B) return __fmul2_rn(ldg2(p.bz + id), u);
+    if (MODE == PML_B) return lp < 2 * R || b_on(z - R) ? __fmul2_rn(ldg2(p.bz + id), u) : z2;
     if (!(layx || layy || layz(z)) || z < 0 || z >= p.nz) return z2;
     return ld2(p.ph[2] + fo + id);
   };
@@ -229,7 +231,7 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
       if (edge(z)) o.q = ld2(p.q + fo + id);
     }
     if (MODE != PML_PHI) o.up = ld2(p.up + fo + id);
-    if (MODE == PML_U && VD) {
+    if (MODE == PML_U && VD && b_on(z)) {
       o.bx = ldg2(p.bx + id);
       o.by = ldg2(p.by + id);
       o.bz = ldg2(p.bz + id);
@@ -271,7 +273,7 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
         float2 acc = z2, dx = z2, dy = z2, dz = z2;   // L u (lap), D1 u (unscaled)
         const float2 cen = RING ? q[RING ? s + R : 0] : z2;
         constexpr bool LAP = MODE == PML_U || MODE == PML_B;
-        const bool d1 = MODE == PML_PHI || (MODE == PML_U && VD) || (MODE == PML_B && lay);
+        const bool d1 = MODE == PML_PHI || (MODE == PML_U && VD && b_on(z)) || (MODE == PML_B && lay);
         float2 X[2 * M + 1], Yp[R + 1], Ym[R + 1];
         if (RING) {
 #pragma unroll
@@ -308,7 +310,7 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
             dy = __fmul2_rn(dy, bc2(p.ih1[1]));
             dz = __fmul2_rn(dz, bc2(p.ih1[2]));
           }
-          if (MODE == PML_U && VD) {
+          if (MODE == PML_U && VD && b_on(z)) {
             float2 t = __fmul2_rn(cur.bx, dx);
             t = __ffma2_rn(cur.by, dy, t);
             t = __ffma2_rn(cur.bz, dz, t);
@@ -485,7 +487,7 @@ k_pml3x(const StepParams p, const __grid_constant__ CUtensorMap xmap,
             put(p.q, idx, make_float2(qb.x - (yz8 * Ax.x) * c.x, qb.y - (yz8 * Ax.y) * c.y));
           }
         } else {   // PML_B
-          if (VD) acc = __fadd2_rn(acc, __fadd2_rn(__fadd2_rn(sx, sy), sz));
+          if (VD && stz) acc = __fadd2_rn(acc, __fadd2_rn(__fadd2_rn(sx, sy), sz));
           put(p.up, idx, __fadd2_rn(cur.up, acc));
           if (lay) {
             const float rz = __frcp_rn(1.f + Az), pzf = p_of(Az);

@@ -665,7 +665,7 @@ void fwi_plan_destroy(fwi_plan* P) {
   if (!P) return;
   cudaSetDevice(P->device);
   for (void* q : {(void*)P->arena, (void*)P->tab, (void*)P->spx, (void*)P->spy, (void*)P->spz,
-                  (void*)P->d_stats, (void*)P->d_flags, (void*)P->d_J})
+                  (void*)P->bflag, (void*)P->d_stats, (void*)P->d_flags, (void*)P->d_J})
     if (q) cudaFreeAsync(q, P->st);
   cudaStreamSynchronize(P->st);
   cudaGetLastError();

@@ -9,6 +9,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 namespace fwi {
 
 namespace {
@@ -47,6 +49,28 @@ struct GeoX2 {
   static constexpr int NOS = 4;             // operand stages: two loop trips
 };
 
+// The planes of a column's chunk on which some density gradient matters to it (bit i:
+// plane z0 + i), from the flags of launch_density_flags; every one without them.
+// Every lane of the warp takes part.
+//
+// A model whose density is constant within its tissues has gradients only near
+// their boundaries.  Elsewhere the variable-density terms add exact zeros, so a
+// plane without any leaves out their loads (24 of some 72 bytes per point of a
+// gradient step pair) and their half of the arithmetic.
+__device__ __forceinline__ unsigned long long density_planes(const StepParams& p, int z0, int nz_c) {
+  if (!p.bflag) return ~0ull;
+  const int lane = threadIdx.x & 31;
+  const long long at = (long long)blockIdx.y * gridDim.x + blockIdx.x, plane = (long long)gridDim.x * gridDim.y;
+  unsigned w[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = 32 * h + lane;
+    const int f = i < nz_c ? __ldg(p.bflag + (z0 + i) * plane + at) : 0;
+    w[h] = __ballot_sync(0xffffffffu, f != 0);
+  }
+  return (unsigned long long)w[1] << 32 | w[0];
+}
+
 // MODE: X2_LEAP the leapfrog, or an extended scheme (ExtMode, fwi_internal.cuh):
 // the plane ring holds the stencil input (u^n, lambda^k, the k w / k L^T lambda
 // scratch, or att lambda), and the update writes k (L x + s) (EXT_KW), the
@@ -58,7 +82,8 @@ constexpr float X2_INV12 = 1.f / 12.f;   // the fourth-order scheme's 1/12, roun
 // CROWD: the injection tables have planes of more than 32 entries in a tile
 // (the 64-node rows of sinc points), whose threads find their own pair's
 // entries by bisection (a separate instantiation).
-template <int R, bool VD, bool ADJ, int BY, int MODE = X2_LEAP, bool CROWD = false>
+// PP: density terms only on the planes that p.bflag marks.
+template <int R, bool VD, bool ADJ, int BY, int MODE = X2_LEAP, bool CROWD = false, bool PP = false>
 __global__ void __launch_bounds__(32 * BY, ((VD && ADJ) ? 512 : 768) / (32 * BY))
 k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
             const __grid_constant__ CUtensorMap bxmap, const __grid_constant__ CUtensorMap bymap,
@@ -114,6 +139,8 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
   // Source entries of the tile are sorted by tile-local index, which grows
   // with the plane: s_pe[lz] = first entry of plane lz (binary search), so a
   // plane's entries are s_pe[lz] .. s_pe[lz + 1] - 1.
+  const unsigned long long bon = PP ? density_planes(p, z0, nz_c) : 0ull;
+  auto b_on = [&](int i) { return !PP || ((bon >> i) & 1) != 0; };   // plane i has density gradients
   bool has_inj = false;
   if (p.inj_off) {
     const int t = b * p.ntiles + (zc * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -156,6 +183,17 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
       tma_load_4d(o + 3 * G::OPT, &opg, &obar[st], xx, yy, zz, b);
     }
   };
+  auto issue_b = [&](int i) {   // b_x, b_y of plane i of the chunk, or nothing if they are zero
+    const int k = i % NBS;
+    if (!b_on(i)) {
+      mbar_arrive(&bbar[k]);
+      return;
+    }
+    float* st = bring + k * G::BSTAGE;
+    mbar_arrive_expect_tx(&bbar[k], G::BSTAGE_BYTES);
+    tma_load_4d(st, &bxmap, &bbar[k], tmx, y0 + p.oy, z0 + i + p.oz, 0);
+    tma_load_4d(st + G::BXB, &bymap, &bbar[k], x0 + p.ox, tmy, z0 + i + p.oz, 0);
+  };
   if (tid == 0) {
     if (OPS)
       for (int ii = 0; ii < NOS && ii < nz_c; ++ii) issue_ops(ii);
@@ -163,14 +201,8 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
       mbar_arrive_expect_tx(&bar[lp], G::PLANE_BYTES);
       tma_load_4d(ring + lp * G::PLANE, &umap, &bar[lp], tmx, tmy, pz0 + lp, b);
     }
-    if (PSI) {
-      for (int i = 0; i < NBS && i < nz_c; ++i) {
-        float* st = bring + i * G::BSTAGE;
-        mbar_arrive_expect_tx(&bbar[i], G::BSTAGE_BYTES);
-        tma_load_4d(st, &bxmap, &bbar[i], tmx, y0 + p.oy, z0 + i + p.oz, 0);
-        tma_load_4d(st + G::BXB, &bymap, &bbar[i], x0 + p.ox, tmy, z0 + i + p.oz, 0);
-      }
-    }
+    if (PSI)
+      for (int i = 0; i < NBS && i < nz_c; ++i) issue_b(i);
   }
 
   const int c0 = G::XOFF + 2 * tx;          // own pair's column in a staged row (even)
@@ -244,7 +276,7 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
     if (LCM || (A2M && !ADJ)) o.x[0] = *reinterpret_cast<const float2*>(p.q + fo + id);
     if (A2M && ADJ) o.x[0] = *reinterpret_cast<const float2*>(p.hist2 + fo + id);
     if (PSI) {   // lambda^{k+1}, k, h, g come from the operand stages
-      o.bzl = ldg2(p.bz + (long long)(pz0 + ii + 2 * R) * p.sxy + col);
+      if (b_on(ii)) o.bzl = ldg2(p.bz + (long long)(pz0 + ii + 2 * R) * p.sxy + col);
       return o;
     }
     if (!OPS && !LCM) {   // (OPS: u^{n-1} and k come from the operand stages)
@@ -255,12 +287,11 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
       o.hv = __ldcs(reinterpret_cast<const float2*>(p.hist + fo + id));
       o.gv = *reinterpret_cast<const float2*>(p.g + fo + id);
     }
-    if (VD && !ADJ) {
+    if (VD && !ADJ && b_on(ii)) {
       o.bx = ldg2(p.bx + id);
       o.by = ldg2(p.by + id);
       o.bz = ldg2(p.bz + id);
     }
-    if (PSI) o.bzl = ldg2(p.bz + (long long)(pz0 + ii + 2 * R) * p.sxy + col);
     return o;
   };
   Ops nxt = load_ops(0);
@@ -283,84 +314,92 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
         const float* cp = ring + ((i + R) % NSU) * G::PLANE;   // centre plane z
         const float* bxp = bring + (i % NBS) * G::BSTAGE;   // b_x rows of the tile
         const float* byp = bxp + G::BXB;                    // b_y columns with the y halo
-        if (PSI && !mbar_wait_bounded(&bbar[i % NBS], (uint32_t)((i / NBS) & 1))) timed_out = true;
+        if (PSI && b_on(i) && !mbar_wait_bounded(&bbar[i % NBS], (uint32_t)((i / NBS) & 1))) timed_out = true;
 
-        // x pairs of the centre row: columns c0 - 2M .. c0 + 2M + 1
-        float2 X[2 * M + 1];
-#pragma unroll
-        for (int k = 0; k <= 2 * M; ++k) X[k] = lds2(cp + (ty + R) * BXW + c0 - 2 * M + 2 * k);
-        auto ux = [&](int d) {   // u at column c0 + d
-          const int e = d + 2 * M;
-          return (e & 1) ? X[e >> 1].y : X[e >> 1].x;
-        };
-        float2 Yp[R + 1], Ym[R + 1];
-#pragma unroll
-        for (int j = 1; j <= R; ++j) {
-          Yp[j] = lds2(cp + (ty + R + j) * BXW + c0);
-          Ym[j] = lds2(cp + (ty + R - j) * BXW + c0);
-        }
-
-        // zero-sum second derivatives per axis, sum_j w_j (u_{+j} + u_{-j} - 2 u_0),
-        // with the unscaled weights as immediates; 1/h^2 applied per axis
         const float2 cen = q[s + R];
-        const float2 n2 = make_float2(-(cen.x + cen.x), -(cen.y + cen.y));
         const float2 z2 = make_float2(0.f, 0.f);
-        float2 ax = z2, ay = z2, az = z2;
+        float2 lap2;
+        // L x of the pair; one copy with the density terms and one without, so that
+        // each schedules its shared-memory reads as one block
+        auto stencil = [&](auto with_b) {
+          constexpr bool on = decltype(with_b)::value;
+          // x pairs of the centre row: columns c0 - 2M .. c0 + 2M + 1
+          float2 X[2 * M + 1];
 #pragma unroll
-        for (int j = 1; j <= R; ++j) {
-          const float2 xp = make_float2(ux(j), ux(j + 1));
-          const float2 xm = make_float2(ux(-j), ux(1 - j));
-          ax = __ffma2_rn(bc2(w2c<R>(j)), __fadd2_rn(__fadd2_rn(xp, xm), n2), ax);
-          ay = __ffma2_rn(bc2(w2c<R>(j)), __fadd2_rn(__fadd2_rn(Yp[j], Ym[j]), n2), ay);
-          az = __ffma2_rn(bc2(w2c<R>(j)),
-                          __fadd2_rn(__fadd2_rn(q[s + R + j], q[s + R - j]), n2), az);
-        }
-        float2 acc = __fmul2_rn(ax, bc2(p.ih2[0]));
-        acc = __ffma2_rn(ay, bc2(p.ih2[1]), acc);
-        acc = __ffma2_rn(az, bc2(p.ih2[2]), acc);
-        const float2 lap2 = acc;   // y = 2: the plain Laplacian
-        if (VD && !ADJ) {
-          float2 dx = z2, dy = z2, dz = z2;
+          for (int k = 0; k <= 2 * M; ++k) X[k] = lds2(cp + (ty + R) * BXW + c0 - 2 * M + 2 * k);
+          auto ux = [&](int d) {   // u at column c0 + d
+            const int e = d + 2 * M;
+            return (e & 1) ? X[e >> 1].y : X[e >> 1].x;
+          };
+          float2 Yp[R + 1], Ym[R + 1];
+#pragma unroll
+          for (int j = 1; j <= R; ++j) {
+            Yp[j] = lds2(cp + (ty + R + j) * BXW + c0);
+            Ym[j] = lds2(cp + (ty + R - j) * BXW + c0);
+          }
+
+          // zero-sum second derivatives per axis, sum_j w_j (u_{+j} + u_{-j} - 2 u_0),
+          // with the unscaled weights as immediates; 1/h^2 applied per axis
+          const float2 n2 = make_float2(-(cen.x + cen.x), -(cen.y + cen.y));
+          float2 ax = z2, ay = z2, az = z2;
 #pragma unroll
           for (int j = 1; j <= R; ++j) {
             const float2 xp = make_float2(ux(j), ux(j + 1));
             const float2 xm = make_float2(ux(-j), ux(1 - j));
-            dx = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(xp, neg2(xm)), dx);
-            dy = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(Yp[j], neg2(Ym[j])), dy);
-            dz = __ffma2_rn(bc2(w1c<R>(j)),
-                            __fadd2_rn(q[s + R + j], neg2(q[s + R - j])), dz);
+            ax = __ffma2_rn(bc2(w2c<R>(j)), __fadd2_rn(__fadd2_rn(xp, xm), n2), ax);
+            ay = __ffma2_rn(bc2(w2c<R>(j)), __fadd2_rn(__fadd2_rn(Yp[j], Ym[j]), n2), ay);
+            az = __ffma2_rn(bc2(w2c<R>(j)),
+                            __fadd2_rn(__fadd2_rn(q[s + R + j], q[s + R - j]), n2), az);
           }
-          float2 t = __fmul2_rn(cur.bx, __fmul2_rn(dx, bc2(p.ih1[0])));
-          t = __ffma2_rn(cur.by, __fmul2_rn(dy, bc2(p.ih1[1])), t);
-          t = __ffma2_rn(cur.bz, __fmul2_rn(dz, bc2(p.ih1[2])), t);
-          acc = __fadd2_rn(acc, neg2(t));
-        }
-        if (PSI) {
-          // b_x lambda on the centre row, b_y lambda on the centre column
-          float2 PX[2 * M + 1];
+          float2 acc = __fmul2_rn(ax, bc2(p.ih2[0]));
+          acc = __ffma2_rn(ay, bc2(p.ih2[1]), acc);
+          acc = __ffma2_rn(az, bc2(p.ih2[2]), acc);
+          lap2 = acc;   // y = 2: the plain Laplacian
+          if (VD && !ADJ && on) {
+            float2 dx = z2, dy = z2, dz = z2;
 #pragma unroll
-          for (int k = 0; k <= 2 * M; ++k)
-            PX[k] = __fmul2_rn(lds2(bxp + ty * BXW + c0 - 2 * M + 2 * k), X[k]);
-          auto px = [&](int d) {
-            const int e = d + 2 * M;
-            return (e & 1) ? PX[e >> 1].y : PX[e >> 1].x;
-          };
-          float2 sx = z2, sy = z2, sz = z2;
-#pragma unroll
-          for (int j = 1; j <= R; ++j) {
-            const float2 pp = make_float2(px(j), px(j + 1));
-            const float2 pm = make_float2(px(-j), px(1 - j));
-            sx = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(pp, neg2(pm)), sx);
-            const float2 yb = __fmul2_rn(lds2(byp + (ty + R + j) * G::TXP + c0 - G::XOFF), Yp[j]);
-            const float2 ya = __fmul2_rn(lds2(byp + (ty + R - j) * G::TXP + c0 - G::XOFF), Ym[j]);
-            sy = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(yb, neg2(ya)), sy);
-            sz = __ffma2_rn(bc2(w1c<R>(j)),
-                            __fadd2_rn(qz[s + R + j], neg2(qz[s + R - j])), sz);
+            for (int j = 1; j <= R; ++j) {
+              const float2 xp = make_float2(ux(j), ux(j + 1));
+              const float2 xm = make_float2(ux(-j), ux(1 - j));
+              dx = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(xp, neg2(xm)), dx);
+              dy = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(Yp[j], neg2(Ym[j])), dy);
+              dz = __ffma2_rn(bc2(w1c<R>(j)),
+                              __fadd2_rn(q[s + R + j], neg2(q[s + R - j])), dz);
+            }
+            float2 t = __fmul2_rn(cur.bx, __fmul2_rn(dx, bc2(p.ih1[0])));
+            t = __ffma2_rn(cur.by, __fmul2_rn(dy, bc2(p.ih1[1])), t);
+            t = __ffma2_rn(cur.bz, __fmul2_rn(dz, bc2(p.ih1[2])), t);
+            acc = __fadd2_rn(acc, neg2(t));
           }
-          acc = __ffma2_rn(sx, bc2(p.ih1[0]), acc);
-          acc = __ffma2_rn(sy, bc2(p.ih1[1]), acc);
-          acc = __ffma2_rn(sz, bc2(p.ih1[2]), acc);
-        }
+          if (PSI && on) {
+            // b_x lambda on the centre row, b_y lambda on the centre column
+            float2 PX[2 * M + 1];
+#pragma unroll
+            for (int k = 0; k <= 2 * M; ++k)
+              PX[k] = __fmul2_rn(lds2(bxp + ty * BXW + c0 - 2 * M + 2 * k), X[k]);
+            auto px = [&](int d) {
+              const int e = d + 2 * M;
+              return (e & 1) ? PX[e >> 1].y : PX[e >> 1].x;
+            };
+            float2 sx = z2, sy = z2, sz = z2;
+#pragma unroll
+            for (int j = 1; j <= R; ++j) {
+              const float2 pp = make_float2(px(j), px(j + 1));
+              const float2 pm = make_float2(px(-j), px(1 - j));
+              sx = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(pp, neg2(pm)), sx);
+              const float2 yb = __fmul2_rn(lds2(byp + (ty + R + j) * G::TXP + c0 - G::XOFF), Yp[j]);
+              const float2 ya = __fmul2_rn(lds2(byp + (ty + R - j) * G::TXP + c0 - G::XOFF), Ym[j]);
+              sy = __ffma2_rn(bc2(w1c<R>(j)), __fadd2_rn(yb, neg2(ya)), sy);
+              sz = __ffma2_rn(bc2(w1c<R>(j)),
+                              __fadd2_rn(qz[s + R + j], neg2(qz[s + R - j])), sz);
+            }
+            acc = __ffma2_rn(sx, bc2(p.ih1[0]), acc);
+            acc = __ffma2_rn(sy, bc2(p.ih1[1]), acc);
+            acc = __ffma2_rn(sz, bc2(p.ih1[2]), acc);
+          }
+          return acc;
+        };
+        float2 acc = !PP || b_on(i) ? stencil(std::true_type()) : stencil(std::false_type());
         if (has_inj) {
           const int lz = z - z0;
           const int l0 = lz * (TY * G::TXP) + loc0;
@@ -522,13 +561,8 @@ k_step3d_x2(const StepParams p, const __grid_constant__ CUtensorMap umap,
             issue_ops(i + NOS);
           }
           if (PSI && i + NBS < nz_c) {
-            const int st = i % NBS;
-            const int zb = z0 + i + NBS + p.oz;
-            float* sb = bring + st * G::BSTAGE;
             fence_proxy_async_smem();
-            mbar_arrive_expect_tx(&bbar[st], G::BSTAGE_BYTES);
-            tma_load_4d(sb, &bxmap, &bbar[st], tmx, y0 + p.oy, zb, 0);
-            tma_load_4d(sb + G::BXB, &bymap, &bbar[st], x0 + p.ox, tmy, zb, 0);
+            issue_b(i + NBS);
           }
         }
       }
