@@ -591,10 +591,9 @@ def roofline(acc, steps, ms, vd, ndim, tile, scheme=""):
     ext = scheme in ("t4", "att0", "att2", "pml")
     if ext:
         bpu = SCHEME_BYTES[(scheme, kind)] + (4 if vd else 0)   # + ln rho
-        # 2D sponge-boundary schemes run on the TMA shot-loop kernels
-        kern = ("k_pml%dd" % ndim if scheme == "pml" else
-                "k_step2d_tma_ext" if ndim == 2 else
-                "k_step3d_x2" if scheme in ("t4", "att0") else "k_ext3d")
+        # 2D on the TMA shot-loop kernels, 3D on the two-point plane rings
+        kern = ("k_step2d_tma_ext + k_pml2d" if scheme == "pml" else "k_step2d_tma_ext") if ndim == 2 else (
+            "k_pml3x" if scheme == "pml" else "k_step3d_x2")
         kname = "%s %s step (%s)" % (kern, "adjoint+imaging" if kind == "adj" else "forward+store",
                                      scheme)
     else:
