@@ -309,7 +309,7 @@ size_t fixed_bytes(const fwi_plan* P, const fwi_geometry* g, bool vd, int B, con
 fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc);
 fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
                        bool split = false, const Scheme& sc = Scheme());
-constexpr double GROUP_TAIL = 0.55;   // the leapfrog's
+constexpr double GROUP_TAIL = 0.55;   // (the PML's: 0.75)
 int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail = GROUP_TAIL);
 int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc);
 int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, int B);

@@ -343,14 +343,15 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc) {
 // Shots per CTA (S) of a 2D per-step launch over problems of (tiles, shots).  In
 // shot times, a CTA of S shots takes about S + 1 (the model loads and the gradient
 // update cost one), two CTAs per SM work at a time, and `tail` of a CTA is waited
-// for at the end of the step: about half, more in the extended schemes, whose CTAs
-// differ (the PML's 1024 x 1024 gradient of 6 shots: S = 3 27.3 ms, S = 6 29.0 ms).
-// The S with the least of the sum is taken.
+// for at the end of the step: about half, more with the PML, whose CTAs differ (its
+// 1024 x 1024 gradient of 6 shots: S = 3 27.3 ms, S = 6 29.0 ms).  The S with the least
+// of the sum is taken.
 // Measured against the largest S <= 6 that leaves four waves of CTAs, us per
 // gradient step pair (8th order, density): 456 x 485, 16 shots 50.8 -> 39.8; 700 x
 // 748, 6 shots 43.3 -> 32.8, 10 shots 70.0 -> 47.9; 1024 x 1024, 6 shots 62.9 ->
 // 56.7, 8 shots 80.0 -> 74.9, 15 shots 132.9 -> 128.6; 1600 x 1600, 16 shots 333.9 ->
-// 311.4; 6 shots of the fourth-order scheme (800 x 872) 80.6 -> 76.1, of the PML
+// 311.4; fourth-order scheme, 6 shots (800 x 872) 80.6 -> 76.1, 15 shots
+// (1024 x 1024) 246.1 -> 243.8; 6 shots of the PML
 // (1024 x 1024) 106.8 -> 103.9.
 int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail) {
   int most = 1, best = 1;
@@ -369,7 +370,7 @@ int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, dou
 }
 
 int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc) {
-  return shot_group(P->nsm, {{tile_geo(P, shape, true).ntiles(), B}}, sc.ext() ? 0.75 : GROUP_TAIL);
+  return shot_group(P->nsm, {{tile_geo(P, shape, true).ntiles(), B}}, sc.pml ? 0.75 : GROUP_TAIL);
 }
 
 // Planes per CTA of the default 3D variant.  A CTA spends about zc + 4 plane
