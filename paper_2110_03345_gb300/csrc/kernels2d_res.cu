@@ -576,8 +576,10 @@ __global__ void __launch_bounds__(32 * RES_WARPS, 1) k_res2d(const ResParams p) 
         nv[e] = __ldg(p.inj_w + eb + e) * p.vals[p.inj_vidx[eb + e] + p.voff + (it + 1) * p.vstep];
     }
   }
-  // A launch of one step has received nothing yet: wait for the neighbours'
-  // words, so that no tile is written back before its neighbours have read it.
+  // A launch of one step has received nothing yet: wait for the neighbours' words,
+  // so that no tile is written back before its neighbours have read it (a word is
+  // sent after its tile is staged).  Each thread waits for its own cells only, hence
+  // the barrier; longer launches have passed one behind the receive of their steps.
   if (p.steps == 1) {
     bool ok = true;
     if (PH == 2) {
@@ -586,7 +588,11 @@ __global__ void __launch_bounds__(32 * RES_WARPS, 1) k_res2d(const ResParams p) 
     }
 #pragma unroll
     for (int ph = 0; ph < PH; ++ph) ok = receive(ph, s_u1, 1u, p.tag0 + 1, ahead, false) && ok;
-    if (!ok && p.flags) atomicOr(p.flags, 2);
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0 && p.flags) atomicOr(p.flags, 2);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      return;
+    }
   }
   // ---- state back to global memory: u^{n+steps} and u^{n+steps-1}
   const float4* fu = (p.steps & 1) ? s_u1 : s_u0;
