@@ -285,7 +285,7 @@ fwi_status build_source_sampling(Call& c, int shot0, int nb, int* d_node, float*
           for (int a = 0; a < 3; ++a) node3[3 * (pt * c.ncorner + q) + a] = ps.node[3 * q + a];
       }
     }
-  if (c.pl.res.on) FWI_TRY(res_sample_table(c, node3, c.pl.B, res, &c.wsmp));
+  if (c.pl.res.on) FWI_TRY(res_sample_table(c, node3, nb, res, &c.wsmp));   // (the last batch has fewer shots than slots)
   // pageable sources: the copies have staged them when cudaMemcpyAsync returns
   CUDA_TRY(cudaMemcpyAsync(d_node, node.data(), node.size() * 4, cudaMemcpyHostToDevice, P->st));
   CUDA_TRY(cudaMemcpyAsync(d_w, w.data(), w.size() * 4, cudaMemcpyHostToDevice, P->st));
