@@ -8,6 +8,8 @@
 
 #include <math.h>
 
+#include <algorithm>
+
 namespace fwi {
 
 namespace {
@@ -92,25 +94,28 @@ __global__ void k_density_grad(Layout L, const float* __restrict__ lnr, AxisW wx
   }
 }
 
-// Flags of one plane of one column tile: 1 b_x is non-zero on its rows with their
-// halo or b_y on its columns with theirs, 2 b_z at its points.
+// Flags of the planes of one column tile: 1 b_x is non-zero on the tile's rows with their
+// halo or b_y on its columns with theirs, 2 b_z at its points.  A block takes every
+// gridDim.z-th plane (a grid may have more planes than a launch has blocks along z).
 __global__ void k_density_plane(Layout L, const float* __restrict__ bx, const float* __restrict__ by,
                                 const float* __restrict__ bz, int rows, unsigned char* __restrict__ flags) {
-  const int x0 = blockIdx.x * 64, y0 = blockIdx.y * rows, z = blockIdx.z;
+  const int x0 = blockIdx.x * 64, y0 = blockIdx.y * rows;
   const int R = L.R, w = 64 + 2 * R, n = w * (rows + 2 * R);
-  int bits = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int dy = i / w - R, dx = i % w - R;
-    const int x = x0 + dx, y = y0 + dy;
-    if (x < 0 || x >= L.nx || y < 0 || y >= L.ny) continue;
-    const bool row = dy >= 0 && dy < rows, col = dx >= 0 && dx < 64;
-    const long long pi = L.index(z, y, x);
-    if ((row && bx[pi] != 0.f) || (col && by[pi] != 0.f)) bits |= 1;
-    if (row && col && bz[pi] != 0.f) bits |= 2;
+  for (int z = blockIdx.z; z < L.nz; z += gridDim.z) {
+    int bits = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int dy = i / w - R, dx = i % w - R;
+      const int x = x0 + dx, y = y0 + dy;
+      if (x < 0 || x >= L.nx || y < 0 || y >= L.ny) continue;
+      const bool row = dy >= 0 && dy < rows, col = dx >= 0 && dx < 64;
+      const long long pi = L.index(z, y, x);
+      if ((row && bx[pi] != 0.f) || (col && by[pi] != 0.f)) bits |= 1;
+      if (row && col && bz[pi] != 0.f) bits |= 2;
+    }
+    const bool any1 = __syncthreads_or(bits & 1), any2 = __syncthreads_or(bits & 2);
+    if (threadIdx.x == 0)
+      flags[((long long)z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = (any1 ? 1 : 0) | (any2 ? 2 : 0);
   }
-  const bool any1 = __syncthreads_or(bits & 1), any2 = __syncthreads_or(bits & 2);
-  if (threadIdx.x == 0)
-    flags[((long long)z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = (any1 ? 1 : 0) | (any2 ? 2 : 0);
 }
 // 1 also where a plane within R along z has b_z; count += the planes with a flag
 __global__ void k_density_window(int nz, int ncol, int R, unsigned char* __restrict__ flags,
@@ -279,7 +284,7 @@ cudaError_t launch_density_grad(const Layout& L, const float* lnr, const AxisW& 
 cudaError_t launch_density_flags(const Layout& L, const float* bx, const float* by, const float* bz,
                                  int rows, int gx, int gy, unsigned char* flags, unsigned int* count,
                                  cudaStream_t st) {
-  k_density_plane<<<dim3(gx, gy, L.nz), 128, 0, st>>>(L, bx, by, bz, rows, flags);
+  k_density_plane<<<dim3(gx, gy, std::min(L.nz, 65535)), 128, 0, st>>>(L, bx, by, bz, rows, flags);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_density_window<<<(gx * gy + 63) / 64, 64, 0, st>>>(L.nz, gx * gy, L.R, flags, count);
