@@ -13,12 +13,35 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device_once.h"
+
 namespace fwi {
 
 constexpr int OX = 8;          // x padding (floats) before the interior
 constexpr int TILE_X = 128;    // tile width of the 2D kernels (32 threads x float4)
 constexpr int ROUND_Y = 64;    // y (and z) extents are rounded to this
 constexpr int MAX_SLOT_TILES = 1 << 20;
+
+// Lets launches of `kernel` on the current device take `bytes` of dynamic shared memory
+// (0: the most a CTA may have, 227 KB with the kernel's static part), and with `carveout`
+// asks for the largest shared-memory share of the L1.
+template <class K>
+cudaError_t allow_smem(DeviceOnce& once, K* kernel, int bytes, bool carveout = false) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || once.done(dev)) return e;
+  if (bytes == 0) {
+    cudaFuncAttributes fa{};
+    e = cudaFuncGetAttributes(&fa, kernel);
+    bytes = 227 * 1024 - (int)fa.sharedSizeBytes;
+  }
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && carveout)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             (int)cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess) once.mark(dev);
+  return e;
+}
 
 struct Layout {
   int ndim;

@@ -288,13 +288,9 @@ template <int R, bool VD, bool ADJ, int RY, int BY>
 cudaError_t launch_t(const StepParams& p, cudaStream_t st) {
   constexpr int TY = RY * BY;
   constexpr size_t smem = smem_bytes<R, VD, ADJ, RY, BY>();
-  static bool attr_set = false;   // per instantiation; set once per process
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step2d<R, VD, ADJ, RY, BY>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step2d<R, VD, ADJ, RY, BY>, (int)smem);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + TILE_X - 1) / TILE_X, (p.ny + TY - 1) / TY, p.B);
   dim3 block(32, BY);
   k_step2d<R, VD, ADJ, RY, BY><<<grid, block, smem, st>>>(p);
@@ -325,13 +321,9 @@ template <int R, bool VD>
 cudaError_t launch_multi_t(const MultiDesc* descs, const MultiUnit* units, int nunits, int n,
                            cudaStream_t st) {
   constexpr size_t smem = smem_bytes<R, VD, false, 4, 8>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step2d_multi<R, VD, 4, 8>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step2d_multi<R, VD, 4, 8>, (int)smem);
+  if (attr != cudaSuccess) return attr;
   if (nunits <= 0) return cudaSuccess;
   k_step2d_multi<R, VD, 4, 8><<<nunits, dim3(32, 8), smem, st>>>(descs, units, n);
   return cudaGetLastError();

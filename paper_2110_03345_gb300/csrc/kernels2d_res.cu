@@ -647,16 +647,10 @@ __global__ void k_res_combine(const float* __restrict__ raw, int nraw, int nslot
 template <int R, bool VD, bool ADJ, int PH, int RY>
 cudaError_t launch_t(const ResParams& p, int nty, int nslots, cudaStream_t st) {
   const size_t smem = res2d_smem(R, VD, ADJ, p.TH, p.nval);
-  // the most a CTA may have, once: a plan's own size here would lower the limit under
+  // the most a CTA may have: a plan's own size here would lower the limit under
   // another thread's launch of a larger one
-  static const cudaError_t attr = [] {
-    cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, k_res2d<R, VD, ADJ, PH, RY>);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_res2d<R, VD, ADJ, PH, RY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               227 * 1024 - (int)fa.sharedSizeBytes);
-    return e;
-  }();
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_res2d<R, VD, ADJ, PH, RY>, 0);
   if (attr != cudaSuccess) return attr;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(p.P, nslots);

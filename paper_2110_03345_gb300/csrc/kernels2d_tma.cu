@@ -43,17 +43,9 @@ cudaError_t launch_t(const StepParams& p, const CUtensorMap& map, const CUtensor
                      const CUtensorMap& hmap, cudaStream_t st) {
   constexpr int TY = RY * BY;
   constexpr size_t smem = smem_bytes<R, VD, ADJ, RY, BY, LEAP, true>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step2d_tma<R, VD, ADJ, RY, BY, CROWD>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step2d_tma<R, VD, ADJ, RY, BY, CROWD>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step2d_tma<R, VD, ADJ, RY, BY, CROWD>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + TILE_X - 1) / TILE_X, (p.ny + TY - 1) / TY, (p.B + p.S - 1) / p.S);
   dim3 block(32, BY);
   return launch_pdl(k_step2d_tma<R, VD, ADJ, RY, BY, CROWD>, grid, block, smem, st, p, map, upmap,

@@ -37,17 +37,9 @@ k_step2d_tma_ext(const StepParams p, const __grid_constant__ CUtensorMap tmap,
 template <int R, bool VD, bool ADJ, int MODE>
 cudaError_t launch_e(const StepParams& p, const CUtensorMap* const* maps, cudaStream_t st) {
   constexpr size_t smem = smem_bytes<R, VD, ADJ, 1, EXT_BY, MODE, true>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step2d_tma_ext<R, VD, ADJ, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step2d_tma_ext<R, VD, ADJ, MODE>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step2d_tma_ext<R, VD, ADJ, MODE>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + TILE_X - 1) / TILE_X, (p.ny + EXT_BY - 1) / EXT_BY, (p.B + p.S - 1) / p.S);
   return launch_pdl(k_step2d_tma_ext<R, VD, ADJ, MODE>, grid, dim3(32, EXT_BY), smem, st, p,
                     *maps[0], *maps[1], *maps[2], *maps[3], *maps[4]);

@@ -48,17 +48,9 @@ template <int R, bool VD, int RY, int BY, bool UW>
 cudaError_t launch_multi_u(const MultiDesc* descs, const MultiUnit* units, int nunits, int n,
                            const AxisW* w, cudaStream_t st) {
   constexpr size_t smem = smem_bytes<R, VD, false, RY, BY, LEAP, true>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step2d_tma_multi<R, VD, RY, BY, UW>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step2d_tma_multi<R, VD, RY, BY, UW>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step2d_tma_multi<R, VD, RY, BY, UW>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   if (nunits <= 0) return cudaSuccess;
   const AxisW zero{};
   return launch_pdl(k_step2d_tma_multi<R, VD, RY, BY, UW>, dim3(nunits), dim3(32, BY), smem,

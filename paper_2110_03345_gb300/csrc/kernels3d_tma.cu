@@ -305,17 +305,9 @@ template <int R, bool VD, bool ADJ, int BY>
 cudaError_t launch_t(const StepParams& p, const CUtensorMap& um, const CUtensorMap& bxm,
                      const CUtensorMap& bym, cudaStream_t st) {
   constexpr size_t smem = smem_bytes3<R, VD, ADJ, BY>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step3d_tma<R, VD, ADJ, BY>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step3d_tma<R, VD, ADJ, BY>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step3d_tma<R, VD, ADJ, BY>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + 31) / 32, (p.ny + BY - 1) / BY, p.B * p.nzc);
   return launch_pdl(k_step3d_tma<R, VD, ADJ, BY>, grid, dim3(32, BY), smem, st, p, um, bxm, bym);
 }

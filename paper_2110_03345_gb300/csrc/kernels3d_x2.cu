@@ -31,17 +31,9 @@ template <int R, bool VD, bool ADJ, int BY, bool CROWD = false, bool PP = false>
 cudaError_t launch_t(const StepParams& p, const CUtensorMap& um, const CUtensorMap& bxm,
                      const CUtensorMap& bym, const CUtensorMap* const* om, cudaStream_t st) {
   constexpr size_t smem = smem_bytes_x2<R, VD, ADJ, BY>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + 63) / 64, (p.ny + BY - 1) / BY, p.B * p.nzc);
   return launch_pdl(k_step3d_x2<R, VD, ADJ, BY, X2_LEAP, CROWD, PP>, grid, dim3(32, BY), smem, st, p,
                     um, bxm, bym, *om[0], *om[1], *om[2], *om[3]);

@@ -20,17 +20,9 @@ constexpr int EXT3_BY = 8;
 template <int R, bool VD, bool ADJ, int MODE, bool PP = false>
 cudaError_t launch_e3(const StepParams& p, const CUtensorMap* const* m, cudaStream_t st) {
   constexpr size_t smem = smem_bytes_x2<R, VD, ADJ, EXT3_BY, MODE>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + 63) / 64, (p.ny + EXT3_BY - 1) / EXT3_BY, p.B * p.nzc);
   return launch_pdl(k_step3d_x2<R, VD, ADJ, EXT3_BY, MODE, false, PP>, grid, dim3(32, EXT3_BY), smem, st, p,
                     *m[0], *m[1], *m[2], *m[3], *m[4], *m[5], *m[6]);

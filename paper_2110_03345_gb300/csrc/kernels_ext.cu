@@ -567,13 +567,9 @@ template <int R, bool VD, bool ADJ, int MODE>
 cudaError_t launch_m(const StepParams& p, int ndim, cudaStream_t st) {
   if (ndim == 2) {
     constexpr size_t smem = Ext2<R, VD, ADJ, MODE>::SMEM;
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaError_t e = cudaFuncSetAttribute(k_ext2d<R, VD, ADJ, MODE>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      attr_set = true;
-    }
+    static DeviceOnce once;
+    const cudaError_t attr = allow_smem(once, k_ext2d<R, VD, ADJ, MODE>, (int)smem);
+    if (attr != cudaSuccess) return attr;
     dim3 grid((p.nx + EXT_TX2 - 1) / EXT_TX2, (p.ny + EXT_TY2 - 1) / EXT_TY2, p.B);
     k_ext2d<R, VD, ADJ, MODE><<<grid, dim3(EXT_TX2 / 4, EXT_TY2), smem, st>>>(p);
   } else {

@@ -531,15 +531,9 @@ template <int R, bool VD, int MODE>
 cudaError_t launch_p(const StepParams& p, const CUtensorMap& xm, const CUtensorMap& rm, const CUtensorMap& cm,
                      cudaStream_t st) {
   constexpr size_t smem = pml_smem<R, VD, MODE>();
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_pml3x<R, VD, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_pml3x<R, VD, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static DeviceOnce once;
+  const cudaError_t attr = allow_smem(once, k_pml3x<R, VD, MODE>, (int)smem, true);
+  if (attr != cudaSuccess) return attr;
   dim3 grid((p.nx + 63) / 64, (p.ny + PB - 1) / PB, p.B * p.nzc);
   return launch_pdl(k_pml3x<R, VD, MODE>, grid, dim3(32, PB), smem, st, p, xm, rm, cm);
 }
