@@ -55,7 +55,7 @@ struct fwi_plan {
   size_t budget = 0;
   cudaStream_t st = nullptr;
   int device = 0;
-  int nsm = 152;            // SM count of the device
+  int nsm = 152;            // SMs of the plan's stream (stream_sms)
   fwi_options opt{};
   fwi_stats stats{};
   fwi::Layout L{};
@@ -290,6 +290,7 @@ struct BatchBufs {
 // ---- plan.cu: plan memory, layout, validation, workspace planning
 cudaError_t pool_alloc(void** ptr, size_t bytes, cudaStream_t st, int device);
 size_t device_available(int device);
+int stream_sms(cudaStream_t st, int device);
 fwi_status ensure_arena(fwi_plan* P, size_t bytes);
 fwi_status ensure_tab(fwi_plan* P, size_t bytes);
 double cfl_limit(int ndim, int order);

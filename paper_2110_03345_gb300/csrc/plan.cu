@@ -102,6 +102,36 @@ fwi_status ensure_tab(fwi_plan* P, size_t bytes) {
   return FWI_OK;
 }
 
+// SMs that launches on a stream may use: those of its context, which are fewer than the
+// device's where the context is a green one.  The resident 2D launches need all of their
+// CTAs on an SM at once, and would be refused with the device's count.
+int stream_sms(cudaStream_t st, int device) {
+  int n = 0;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+    cudaGetLastError();
+    return 152;
+  }
+  auto entry = [](const char* name, unsigned version) -> void* {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return f;
+    cudaGetLastError();
+    return nullptr;
+  };
+  static const auto stream_ctx = reinterpret_cast<PFN_cuStreamGetCtx_v12050>(entry("cuStreamGetCtx", 12050));
+  static const auto ctx_res = reinterpret_cast<PFN_cuCtxGetDevResource_v12040>(entry("cuCtxGetDevResource", 12040));
+  static const auto green_res =
+      reinterpret_cast<PFN_cuGreenCtxGetDevResource_v12040>(entry("cuGreenCtxGetDevResource", 12040));
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r{};
+  if (!stream_ctx || !ctx_res || !green_res || stream_ctx(st, &ctx, &green) != CUDA_SUCCESS) return n;
+  const CUresult e = green ? green_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) : ctx_res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM);
+  return e == CUDA_SUCCESS && r.sm.smCount > 0 ? std::min(n, (int)r.sm.smCount) : n;
+}
+
 double cfl_limit(int ndim, int order) {
   double w2[6], w1[6];
   fd_weights(order, w2, w1);
@@ -604,10 +634,7 @@ fwi_status fwi_plan_create(fwi_plan** plan, const fwi_grid* grid, int nt, double
   if (e != cudaSuccess) return cleanup(fail(FWI_ERR_CUDA, cudaGetErrorString(e)));
   fr = device_available(P->device);   // free memory plus the pool's unused reserve
   P->budget = hbm_budget_bytes ? hbm_budget_bytes : (size_t)(0.9 * (double)fr);
-  if (cudaDeviceGetAttribute(&P->nsm, cudaDevAttrMultiProcessorCount, P->device) != cudaSuccess) {
-    cudaGetLastError();
-    P->nsm = 152;
-  }
+  P->nsm = stream_sms(P->st, P->device);
   {
     // keep freed plan memory cached in the default pool (no return to the OS
     // between requests); this is a per-process allocator setting
