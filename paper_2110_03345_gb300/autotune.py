@@ -7,10 +7,12 @@ device time of every stencil launch from the plan's CUDA events, and keeps the
 variant with the lowest time per step (forward + adjoint for gradients).
 Results are cached in a JSON file keyed by the problem class (dimension,
 order, density mode, grid rounded to the tile sizes, shots per batch), so a
-class is tuned once per machine.
+class is tuned once per machine and version of the kernels.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import os
 import threading
@@ -25,12 +27,30 @@ _lock = threading.Lock()
 CANDIDATES_2D = [dict(tile=t, shots_per_cta=s) for t in (5, 6, 7, 8) for s in (2, 3, 4, 5, 6, 8)] + \
                 [dict(tile=t) for t in (0, 1, 2, 3, 4)]
 CANDIDATES_3D = [dict(tile=t) for t in (5, 6, 7, 8, 9, 10, 11, 12)]
+DEFAULT = dict(tile=0)   # the plan's own choice, which no fixed variant stands for (3D: planes per CTA)
 
 
 def problem_key(shape, order, variable_density, gradient, shots):
     rounded = tuple(int(np.ceil(s / 64.0)) * 64 for s in shape)
     return f"{len(shape)}d-o{order}-{'vd' if variable_density else 'cd'}-" \
            f"{'grad' if gradient else 'fwd'}-{'x'.join(map(str, rounded))}-b{shots}"
+
+
+@functools.lru_cache(maxsize=None)
+def kernels_id():
+    """Digest of the kernel and host sources that the timings were made with."""
+    h = hashlib.sha256()
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    for name in sorted(os.listdir(src)):
+        with open(os.path.join(src, name), "rb") as f:
+            h.update(name.encode() + b"\0" + f.read())
+    return h.hexdigest()[:16]
+
+
+def _cached(cache, key):
+    """Options of a class tuned with the present kernels, or None."""
+    e = cache.get(key)
+    return dict(e["options"]) if e and e.get("kernels") == kernels_id() else None
 
 
 def _load_cache(path):
@@ -60,11 +80,11 @@ def tune(shape, spacing, dt, order, sponge, c_ref, vp, rho, geometry, wavelet, o
     nb = batch or geometry.nshots
     key = problem_key(shape, order, rho is not None, gradient, nb)
     with _lock:
-        cache = _load_cache(cache_path)
-        if not refresh and key in cache:
-            return dict(cache[key]["options"])
+        known = _cached(_load_cache(cache_path), key)
+    if known is not None and not refresh:
+        return known
     if candidates is None:
-        candidates = CANDIDATES_2D if len(shape) == 2 else CANDIDATES_3D
+        candidates = CANDIDATES_2D if len(shape) == 2 else [DEFAULT] + CANDIDATES_3D
     nt = int(min(steps, wavelet.shape[-1]))
     wav = wavelet[..., :nt].contiguous()
     obs = observed[..., :nt].contiguous() if gradient else None
@@ -95,7 +115,7 @@ def tune(shape, spacing, dt, order, sponge, c_ref, vp, rho, geometry, wavelet, o
     best = min(results, key=lambda r: r[0])
     with _lock:
         cache = _load_cache(cache_path)
-        cache[key] = {"options": best[1], "ms_per_step": best[0],
+        cache[key] = {"options": best[1], "ms_per_step": best[0], "kernels": kernels_id(),
                       "tried": [[r[0], r[1]] for r in results]}
         _store_cache(cache_path, cache)
     return dict(best[1])
@@ -123,9 +143,9 @@ def tune_batch(problems, steps=80, candidates=None, cache_path=_CACHE, refresh=F
     time from the batch's events)."""
     key = batch_key(problems)
     with _lock:
-        cache = _load_cache(cache_path)
-        if not refresh and key in cache:
-            return dict(cache[key]["options"])
+        known = _cached(_load_cache(cache_path), key)
+    if known is not None and not refresh:
+        return known
     cut = []
     for pr in problems:
         q = dict(pr)
@@ -152,7 +172,7 @@ def tune_batch(problems, steps=80, candidates=None, cache_path=_CACHE, refresh=F
     best = min(results, key=lambda r: r[0])
     with _lock:
         cache = _load_cache(cache_path)
-        cache[key] = {"options": best[1], "ms_per_run": best[0],
+        cache[key] = {"options": best[1], "ms_per_run": best[0], "kernels": kernels_id(),
                       "tried": [[r[0], r[1]] for r in results]}
         _store_cache(cache_path, cache)
     return dict(best[1])
