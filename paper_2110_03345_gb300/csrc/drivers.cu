@@ -748,7 +748,7 @@ fwi_status finish_call(Call& c) {
     if (c.fwd_launches) s.fwd_ms *= (double)c.fwd_timed / c.fwd_launches;
     if (c.adj_launches) s.adj_ms *= (double)c.adj_timed / c.adj_launches;
   }
-  if (flags[1] & 2) return fail(FWI_ERR_TIMEOUT, "a bounded wait on a TMA copy timed out");
+  if (flags[1] & 2) return fail(FWI_ERR_TIMEOUT, "a bounded wait on a TMA copy or on another CTA's halo timed out");
   if (flags[0]) return fail(FWI_ERR_NONFINITE, "non-finite values in the result (unstable run?)");
   return FWI_OK;
 }

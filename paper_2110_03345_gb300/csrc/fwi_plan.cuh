@@ -175,7 +175,6 @@ struct ResPlan {
   bool on = false;
   int gx = 0, gy = 0, ph = 1, ry = 1, nty = 1, TH = 0, P = 0, conc = 1;
   int nval = 0;         // most injection entries of one CTA
-  int chunk = 1;        // steps per launch at most while samples are taken
   size_t raw = 0;       // floats of the raw sample buffer
   size_t ex = 0;        // 8-byte words of the halo exchange
   size_t inv = 0;       // floats of the sponge's 1 / (1 + a)

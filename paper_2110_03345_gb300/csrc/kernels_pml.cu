@@ -198,10 +198,6 @@ cudaError_t launch_pml2d(const StepParams& p, int R, int mode, cudaStream_t st) 
   return cudaErrorInvalidValue;   // (PML_U and PML_B: EXT_PML of kernels2d_tma_ext.cu)
 }
 
-}  // namespace fwi
-
-namespace fwi {
-
 namespace {
 
 // field[slot][node] += w val for every entry of every (slot, tile) bucket, one

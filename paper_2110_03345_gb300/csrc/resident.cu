@@ -243,8 +243,6 @@ fwi_status res_forward_steps(Call& c, int nb, const DevTable& src, float* A, flo
       ResParams p = res_params(c);
       p.u = p.u_out = A + s0 * fs;
       p.up = p.up_out = Bf + s0 * fs;
-      p.u = A + s0 * fs;
-      p.up = Bf + s0 * fs;
       p.hist = hist ? hist + (size_t)(n - n0) * p.hstride + s0 * fs : nullptr;
       p.inj_off = src.off + (size_t)s0 * r.P;
       p.inj_loc = src.loc;
