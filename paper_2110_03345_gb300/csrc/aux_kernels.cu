@@ -117,20 +117,20 @@ __global__ void k_density_plane(Layout L, const float* __restrict__ bx, const fl
       flags[((long long)z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = (any1 ? 1 : 0) | (any2 ? 2 : 0);
   }
 }
-// 1 also where a plane within R along z has b_z; count += the planes with a flag
-__global__ void k_density_window(int nz, int ncol, int R, unsigned char* __restrict__ flags,
-                                 unsigned int* __restrict__ count) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncol) return;
-  unsigned int n = 0;
-  int last = -R - 1;   // the newest plane with b_z, looking R ahead
-  for (int z = 0; z < nz + R; ++z) {
-    if (z < nz && (flags[(long long)z * ncol + c] & 2)) last = z;
-    const int t = z - R;
-    if (t >= 0 && last >= t - R) flags[(long long)t * ncol + c] |= 1;
-    if (t >= 0) n += flags[(long long)t * ncol + c] != 0;
+// flags = raw, and 1 also where a plane within R along z has b_z; count += the planes with a flag
+__global__ void k_density_window(int nz, int ncol, int R, const unsigned char* __restrict__ raw,
+                                 unsigned char* __restrict__ flags, unsigned int* __restrict__ count) {
+  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  int f = 0;
+  if (i < (long long)nz * ncol) {
+    const int z = (int)(i / ncol);
+    f = raw[i];
+    for (int d = max(-R, -z); d <= min(R, nz - 1 - z); ++d)
+      if (raw[i + (long long)d * ncol] & 2) f |= 1;
+    flags[i] = (unsigned char)f;
   }
-  atomicAdd(count, n);
+  const int n = __syncthreads_count(f);
+  if (threadIdx.x == 0 && n) atomicAdd(count, (unsigned)n);
 }
 
 __global__ void k_sample(StepParams p) {
@@ -282,12 +282,13 @@ cudaError_t launch_density_grad(const Layout& L, const float* lnr, const AxisW& 
 }
 
 cudaError_t launch_density_flags(const Layout& L, const float* bx, const float* by, const float* bz,
-                                 int rows, int gx, int gy, unsigned char* flags, unsigned int* count,
-                                 cudaStream_t st) {
-  k_density_plane<<<dim3(gx, gy, std::min(L.nz, 65535)), 128, 0, st>>>(L, bx, by, bz, rows, flags);
+                                 int rows, int gx, int gy, unsigned char* raw, unsigned char* flags,
+                                 unsigned int* count, cudaStream_t st) {
+  k_density_plane<<<dim3(gx, gy, std::min(L.nz, 65535)), 128, 0, st>>>(L, bx, by, bz, rows, raw);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_density_window<<<(gx * gy + 63) / 64, 64, 0, st>>>(L.nz, gx * gy, L.R, flags, count);
+  const long long n = (long long)L.nz * gx * gy;
+  k_density_window<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(L.nz, gx * gy, L.R, raw, flags, count);
   return cudaGetLastError();
 }
 

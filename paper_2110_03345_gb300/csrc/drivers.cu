@@ -577,7 +577,8 @@ fwi_status prepare_model(Call& c) {
     e = launch_density_grad(P->L, c.W.lnr, P->wx, P->wy, P->wz, c.W.bx, c.W.by, c.W.bz, P->st);
     if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
     c.few_b = false;
-    if (c.pl.x2 && !P->fixed_memory) {
+    const long long pts = (long long)P->L.nx * P->L.ny * P->L.nz * c.pl.B;
+    if (c.pl.x2 && !P->fixed_memory && density_flags_pay(pts, P->nt, c.pl.gradient, c.pl.sc.pml)) {
       // the plane rings leave out the density terms where no gradient reaches.  Choosing
       // per plane costs 5% where there is one (forward 152 x 160 x 176, order 10, 300
       // steps: 12.4 ms with every term; gradients everywhere 13.1, nowhere 10.1; adjoint
@@ -585,15 +586,16 @@ fwi_status prepare_model(Call& c) {
       // planes, counted here.
       const int rows = tile3_variant(c.pl.shape).by;
       const int gx = (P->L.nx + 63) / 64, gy = (P->L.ny + rows - 1) / rows;
-      if (!P->bflag && cudaMallocAsync(reinterpret_cast<void**>(&P->bflag),
-                                       (size_t)P->L.nz * ((P->L.ny + 7) / 8) * gx, P->st) != cudaSuccess) {
+      const size_t most = (size_t)P->L.nz * ((P->L.ny + 7) / 8) * gx;   // flags of a plan's call
+      if (!P->bflag && cudaMallocAsync(reinterpret_cast<void**>(&P->bflag), 2 * most, P->st) != cudaSuccess) {
         P->bflag = nullptr;   // (every term then)
         cudaGetLastError();
       }
       if (P->bflag) {
         unsigned int n = 0;
         CUDA_TRY(cudaMemsetAsync(P->d_stats + 8, 0, sizeof(n), P->st));
-        e = launch_density_flags(P->L, c.W.bx, c.W.by, c.W.bz, rows, gx, gy, P->bflag, P->d_stats + 8, P->st);
+        e = launch_density_flags(P->L, c.W.bx, c.W.by, c.W.bz, rows, gx, gy, P->bflag + most, P->bflag,
+                                 P->d_stats + 8, P->st);
         if (e != cudaSuccess) return fail(FWI_ERR_CUDA, cudaGetErrorString(e));
         CUDA_TRY(cudaMemcpyAsync(&n, P->d_stats + 8, sizeof(n), cudaMemcpyDeviceToHost, P->st));
         CUDA_TRY(cudaStreamSynchronize(P->st));

@@ -404,10 +404,11 @@ cudaError_t launch_model_prep(const Layout& L, const float* vp, const float* rho
                               cudaStream_t st);
 // flags[(z * gy + iy) * gx + ix], of the 64 x rows column tiles (gx x gy) and planes:
 // non-zero where the density terms (the adjoint's: b_x within R along x, b_y along y, b_z
-// along z) reach a non-zero b from the tile; count += the flags set
+// along z) reach a non-zero b from the tile; count += the flags set; raw: as many bytes
+// of scratch
 cudaError_t launch_density_flags(const Layout& L, const float* bx, const float* by, const float* bz,
-                                 int rows, int gx, int gy, unsigned char* flags, unsigned int* count,
-                                 cudaStream_t st);
+                                 int rows, int gx, int gy, unsigned char* raw, unsigned char* flags,
+                                 unsigned int* count, cudaStream_t st);
 cudaError_t launch_density_grad(const Layout& L, const float* lnr, const AxisW& wx,
                                 const AxisW& wy, const AxisW& wz, float* bx, float* by,
                                 float* bz, cudaStream_t st);

@@ -5,6 +5,7 @@
 #pragma once
 #include "fwi.h"
 #include "fwi_internal.cuh"
+#include "launch_rules.h"
 
 #include <cudaTypedefs.h>
 
