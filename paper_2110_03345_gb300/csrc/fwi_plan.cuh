@@ -313,7 +313,7 @@ fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool g
 constexpr double GROUP_TAIL = 0.55;   // (the PML's: 0.75)
 int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail = GROUP_TAIL);
 int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc);
-int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, int B);
+int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, bool pml, int B);
 void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Carve& C, Work& W);
 
 // ---- tables.cu: interpolation and injection tables

@@ -2,6 +2,8 @@
 // CUDA types, so that they can be checked without a GPU).
 #pragma once
 
+#include <cmath>
+
 namespace fwi {
 
 // Whether a 3D call makes and uses the density flags (launch_density_flags): `points` grid
@@ -10,12 +12,50 @@ namespace fwi {
 // by the loads and the arithmetic that the flags spare, and lose to the choice per plane.
 // Gain per step (step pair for gradients) with a density that is constant within two
 // tissues, order 10, in us: leapfrog forward 100^3 -0.4, 128^3 -0.2, 152 x 160 x 176 0, 192
-// x 180 x 200 2.5, 256^3 8.4, 384^3 53; gradient -1.8, -1.3, -0.4, 11.8, 20.6, 118; PML
-// forward 64^3 0, 100^3 0.6, 300 x 64 x 64 2.2, 128^3 4.2, 256^3 17; gradient 0, 2.3, 5.8, 5.9,
-// 56.  So the leapfrog takes them from 5.5 million points, the PML from a million, and
-// either where the run is long enough to win their cost back (8-37 steps).
+// x 180 x 200 2.5, 256^3 8.4, 384^3 53; gradient -1.8, -1.3, -0.4, 11.8, 20.6, 118, four shots
+// of 300 x 64 x 64 6.7; PML forward 64^3 0, 100^3 0.6, 300 x 64 x 64 2.2, 128^3 4.2, 256^3 17;
+// gradient 0, 2.3, 5.8, 5.9, 56.  So the leapfrog takes them from 4.5 million points, the
+// PML from a million, and either where the run is long enough to win their cost back
+// (8-37 steps).
 inline bool density_flags_pay(long long points, int nt, bool grad, bool pml) {
-  return points >= (pml ? 1000000LL : 5500000LL) && (grad ? 4LL : 1LL) * nt >= 40;
+  return points >= (pml ? 1000000LL : 4500000LL) && (grad ? 4LL : 1LL) * nt >= 40;
+}
+
+// Planes per CTA of the default 3D variant (0: none fits `most_chunks`), for `cols` column
+// tiles over all slots.  A CTA of zc planes spends about zc + 5 plane times (the 2R halo
+// planes before its first point cost less than computed ones; PML zc + 3, two of its passes
+// have none or few); three share an SM, two in the variable-density adjoint and the PML.
+// With x CTAs per place a launch takes between ceil(x) of these, if all keep step, and x + a
+// tail, if they drift apart: a weighted mean of the two.
+// (Rounds alone, the rule before this one, took a half-empty round of 48 planes at 192
+// planes and 1.84 rounds of 46 at 320.)
+// us per step / step pair, order 10, one shot, 32 planes -> rounds alone -> this rule.  With
+// density: 128^3 45.6 -> 18.8 -> 18.8 / 94.2 -> 51.2 -> 51.2, 152 x 160 x 176 51.4 -> 38.4 -> 38.4 /
+// 103.2 in all, 192 x 180 x 200 68.7 -> 75.8 -> 63.8 / 161.0 -> 158.9 -> 158.9, 256^3 115.7 ->
+// 108.5 -> 108.5 / 282.6 -> 264.1 -> 264.1.  Without: 192 x 180 x 200 67.1 -> 64.5 -> 54.6 / 152.5 ->
+// 142.3 -> 122.1, 96 x 300 x 300 69.3 -> 64.4 -> 57.8 / 157.3 -> 144.1 -> 130.2, 320 x 240 x 200
+// 110.6 -> 116.0 -> 107.4 / 250.2 -> 259.1 -> 242.3.  PML: 192 x 180 x 200 257.4 -> 303.4 -> 213.0 /
+// 537.0 -> 486.6 -> 483.1, 256^3 365.3 -> 363.8 -> 342.3 / 833.7 -> 821.7 -> 803.7.
+inline int z_planes(int nsm, int nz, long long cols, bool vd, bool grad, bool pml, int most_planes,
+                    long long most_chunks) {
+  int best = 0;
+  double least = 0.0;
+  for (int nzc = 1; nzc <= nz && nzc <= most_chunks; ++nzc) {
+    const int zc = (nz + nzc - 1) / nzc;
+    if (zc > most_planes || (nz + zc - 1) / zc != nzc) continue;
+    if (zc < 8 && best > 0) break;
+    auto cost = [&](int per_sm, int halo, double rounds, double tail) {
+      const double x = (double)(cols * nzc) / ((double)per_sm * nsm);
+      return (zc + halo) * (rounds * std::ceil(x) + (1.0 - rounds) * (x + tail));
+    };
+    const double fwd = cost(3, 5, 0.8, 1.3), adj = vd ? cost(2, 5, 0.9, 1.3) : fwd;
+    const double c = pml ? cost(2, 3, 0.6, 1.6) : fwd + (grad ? adj : 0.0);
+    if (best == 0 || c < least) {
+      best = zc;
+      least = c;
+    }
+  }
+  return best;
 }
 
 }  // namespace fwi

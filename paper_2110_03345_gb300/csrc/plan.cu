@@ -403,32 +403,9 @@ int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc) {
   return shot_group(P->nsm, {{tile_geo(P, shape, true).ntiles(), B}}, sc.pml ? 0.75 : GROUP_TAIL);
 }
 
-// Planes per CTA of the default 3D variant.  A CTA spends about zc + 4 plane
-// times (the 2R halo planes before its first point cost less than computed
-// ones), three CTAs share an SM (the variable-density adjoint: two), and a
-// launch takes as many rounds as its CTAs need; the chunk with the fewest
-// plane times over the forward and adjoint launches is taken.  Measured against
-// the fixed 32 planes, us per step (pair): 152 x 160 x 176 forward 62 -> 48,
-// 128^3 forward 47 -> 22 and gradient 97 -> 56, 192^3 gradient 170 -> 165, 256^3
-// gradient 359 -> 337 (37 planes).
-int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, int B) {
-  const int nz = P->L.nz;
-  const long long cols = (long long)T.gx * T.gy * B;
-  int best = T.zc;
-  long long cost = -1;
-  for (int nzc = 1; nzc <= nz; ++nzc) {
-    const int zc = (nz + nzc - 1) / nzc;
-    if (zc > MAX_ZCHUNK || (nz + zc - 1) / zc != nzc) continue;
-    if (zc < 8 && cost >= 0) break;
-    if ((long long)B * nzc > 65535) break;
-    auto rounds = [&](int per_sm) { return (cols * nzc + (long long)per_sm * P->nsm - 1) / ((long long)per_sm * P->nsm); };
-    const long long c = (zc + 4) * (rounds(3) + (grad ? rounds(vd ? 2 : 3) : 0));
-    if (cost < 0 || c < cost) {
-      cost = c;
-      best = zc;
-    }
-  }
-  return best;
+int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, bool pml, int B) {
+  const int zc = z_planes(P->nsm, P->L.nz, (long long)T.gx * T.gy * B, vd, grad, pml, MAX_ZCHUNK, 65535 / B);
+  return zc > 0 ? zc : T.zc;
 }
 
 static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad,
@@ -496,7 +473,7 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
   out.nbatches = (ns + B - 1) / B;
   out.zc = 0;
   if (P->grid.ndim == 3 && P->opt.tile == 0 && out.x2 && !P->fixed_memory)
-    out.zc = z_chunk(P, tile_geo(P, out.shape, out.tma, out.x2), vd || sc.pml, grad, B);
+    out.zc = z_chunk(P, tile_geo(P, out.shape, out.tma, out.x2), vd, grad, sc.pml, B);
   out.S = 1;
   out.res = ResPlan();
   if (resident) choose_res(P, g, vd, grad, B, sc, &out.res);

@@ -18,6 +18,9 @@ int main() {
     auto read = [&](int n) { for (int i = 0; i < n; ++i) if (scanf("%lf", &a[i]) != 1) return false; return true; };
     if (!strcmp(what, "flags") && read(4))
       printf("%d\n", (int)fwi::density_flags_pay((long long)a[0], (int)a[1], a[2] != 0, a[3] != 0));
+    else if (!strcmp(what, "planes") && read(6))   // nz, columns, density, gradient, PML, most chunks
+      printf("%d\n", fwi::z_planes(152, (int)a[0], (long long)a[1], a[2] != 0, a[3] != 0, a[4] != 0, 64,
+                                   (long long)a[5]));
     else return 1;
   }
 }
@@ -62,3 +65,72 @@ def test_density_flags(rules):
             assert net > -20, r
         else:
             assert not (large and nt >= 100), r
+
+
+# us per step (pair) of one shot by planes per CTA, order 10: leapfrog with density (leap) and
+# without (cd), PML; forward and gradient
+Z_TIMES = """
+128 128 128 leap fwd 9:16.2 10:18.8 13:22.7 16:25.9 22:31.6 32:45.6
+128 128 128 leap grad 9:46.5 10:49.3 13:56.9 15:51.2 16:53.2 22:68.9 32:94.2
+128 128 128 cd fwd 9:14 10:16.3 13:19.7 16:22.1 22:27.5 32:38.4
+128 128 128 cd grad 9:30.9 10:35 13:42.4 16:49.1 22:61.4 32:84.8
+128 128 128 pml fwd 9:74.6 10:78.8 13:88.2 16:91.7 22:117.6 32:160.3
+128 128 128 pml grad 8:167.2 10:179.7 13:188.6 15:171.2 16:181.7 22:234.5 32:321.9
+152 160 176 leap fwd 10:37.8 14:40 16:42.2 22:38.4 31:51.4 38:61.1
+152 160 176 leap grad 10:102.9 14:105.7 16:103.3 22:105.2 31:103.2 38:120.5
+152 160 176 cd fwd 10:28.2 14:30.2 16:30.8 22:30.6 31:41.3 38:49.3
+152 160 176 cd grad 10:65.2 14:71.1 16:75.4 22:69.4 31:93.6 38:111.4
+152 160 176 pml fwd 10:129 14:139 16:128.9 22:159.6 31:167 38:199.5
+152 160 176 pml grad 10:292.8 14:308.2 16:292 22:350.8 31:335.8 38:397
+192 180 200 leap fwd 10:64.7 14:62.7 16:65.3 20:62.3 22:63.8 28:66.6 32:68.7 39:77 48:75.8
+192 180 200 leap grad 10:177.3 14:166.5 16:166.6 22:158.9 28:165.2 32:161 39:178
+192 180 200 cd fwd 10:58.7 14:55.8 16:58.7 22:54.6 28:60.6 32:67.1 39:74 48:64.5
+192 180 200 cd grad 10:129 14:124 16:131 22:122.1 28:137.6 32:152.5 39:165.3 48:142.3
+192 180 200 pml fwd 10:215.4 14:211.8 16:227.7 22:219.6 28:246.1 32:257.4 39:263.7 48:303.4
+192 180 200 pml grad 10:497.7 14:484.4 16:507 20:475.8 22:486.6 28:533.5 32:537 39:580
+256 256 256 leap fwd 10:112 14:109.7 16:110.2 22:106.7 29:108.7 32:115.7 37:108.5
+256 256 256 leap grad 10:311.3 14:293.4 16:290.3 22:276.1 29:270.8 32:282.6 37:264.1
+256 256 256 cd fwd 10:100.7 14:100.1 16:99.4 19:93.7 22:98.1 29:95.7 32:102.2 37:94.7
+256 256 256 cd grad 10:226.9 14:228 16:226 22:226.4 29:222.3 32:238.6 37:215.4
+256 256 256 pml fwd 10:332.7 14:331.7 16:342.3 22:325.6 29:344.8 32:365.3 37:363.8
+256 256 256 pml grad 10:806 14:790.3 16:803.7 22:765.4 29:796.5 32:833.7 37:821.7
+96 300 300 leap fwd 10:62.7 14:61.4 16:63.2 20:64.7 32:72.2 48:71
+96 300 300 leap grad 10:180 14:167 16:163 20:167 24:164.8 32:160.2
+96 300 300 cd fwd 10:59.3 14:57.8 16:59.3 20:62.1 24:56.7 32:69.3 48:64.4
+96 300 300 cd grad 10:133.7 14:130.2 16:134.7 20:142.1 32:157.3 48:144.1
+96 300 300 pml fwd 10:205.1 14:214.7 16:225.1 20:217.9 32:257.3 48:306.7
+96 300 300 pml grad 10:484.5 14:490.7 16:497.8 20:490.9 24:522.5 32:531.9
+320 240 200 leap fwd 10:126.4 14:121.8 16:121.4 22:116.8 30:115.4 32:120.8 36:122.7 46:120.7
+320 240 200 leap grad 10:354.2 14:329.3 16:319.8 22:299 30:295.5 32:296 36:300 46:291.8
+320 240 200 cd fwd 10:118.5 14:115.7 16:114 22:112.9 30:107.4 32:110.6 36:117.4 46:116
+320 240 200 cd grad 10:263.2 14:259.2 16:256.5 22:252.6 30:242.3 32:250.2 36:264.6 46:259.1
+320 240 200 pml fwd 10:420.9 14:408.2 16:417.3 22:400 30:407.7 32:434 36:443.2 46:448.7
+320 240 200 pml grad 10:987.9 14:948.9 16:956.6 22:917 30:925.7 32:963.8 36:979 46:987.7
+"""
+
+
+def test_planes_per_cta(rules):
+    """The chosen planes are within 2% of the fixed 32 of before, or faster, and within 17% of
+    the best (small grids, where another chunk hides more latency)."""
+    table = []
+    for line in Z_TIMES.strip().splitlines():
+        f = line.split()
+        table.append((tuple(map(int, f[:3])), f[3], f[4], {int(a): float(b) for a, b in (x.split(":") for x in f[5:])}))
+    picks = rules([("planes", s[0], -(-s[2] // 64) * -(-s[1] // 8), int(m != "cd"), int(k == "grad"), int(m == "pml"),
+                    65535) for s, m, k, _ in table])
+    for (shape, mode, kind, t), z in zip(table, picks):
+        fixed = t[-(-shape[0] // -(-shape[0] // 32))]
+        near = t[min(t, key=lambda q: abs(q - z))]
+        assert near <= 1.02 * fixed and near <= 1.17 * min(t.values()), (shape, mode, kind, z)
+
+
+def test_planes_fit_their_limits(rules):
+    cases = [(nz, cols, vd, grad, pml, most) for nz in (4, 5, 7, 8, 9, 63, 64, 65, 127, 1000, 70001)
+             for cols in (1, 30, 5000) for vd, grad, pml in ((0, 0, 0), (1, 1, 0), (1, 0, 1))
+             for most in (65535, 2000, 1)]
+    for (nz, cols, vd, grad, pml, most), z in zip(cases, rules([("planes", *c) for c in cases])):
+        if z == 0:
+            assert most * 64 < nz                       # no chunk of 64 planes or fewer fits
+        else:
+            chunks = -(-nz // int(z))
+            assert 1 <= z <= 64 and chunks <= most and -(-nz // chunks) == z   # chunks of equal planes
