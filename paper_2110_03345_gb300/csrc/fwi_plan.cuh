@@ -344,7 +344,7 @@ TileGeo call_geo(const fwi_plan* P, const Plan& pl);
 // ---- resident.cu: on-chip 2D runs
 bool res_eligible(const fwi_plan* P, bool grad, int B, const Scheme& sc);
 size_t res_buffers(const fwi_plan* P, const fwi_geometry* g, int B);   // device bytes, B shots at most
-void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, int B, const Scheme& sc,
+void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, int B, int K, const Scheme& sc,
                 ResPlan* out);
 fwi_status res_sample_table(Call& c, const std::vector<int>& nodes3, int slots, Carve& C, ResSamples* out);
 fwi_status res_forward_steps(Call& c, int nb, const DevTable& src, float* A, float* Bf, int n0, int n1,

@@ -58,4 +58,15 @@ inline int z_planes(int nsm, int nz, long long cols, bool vd, bool grad, bool pm
   return best;
 }
 
+// Whether runs of `nt` samples (gradients: between checkpoints every K steps, 0: none) are
+// long enough for resident launches.  A launch loads and stores the whole state and a call
+// clears the exchange buffer, some 20 us each.  One shot with density on 256 x 256, 456 x
+// 485, 700 x 748 and 1024 x 1024, times summed, per-step -> resident: gradient of 200 steps
+// with K = 1 32.1 -> 53.0 ms, 2 22.8 -> 28.9, 4 17.5 -> 18.1, 6 16.1 -> 14.6 (700 x 748 alone 3.9 ->
+// 4.2), 8 15.2 -> 12.7; forward of nt - 1 = 1 747 -> 825 us, 4 802 -> 850, 8 882 -> 890, 16 1020 ->
+// 968; gradient of 2 1032 -> 1111, 8 1315 -> 1256.
+inline bool resident_run(int nt, int K, bool grad) {
+  return grad && K > 0 && K < nt - 1 ? K >= 6 : nt - 1 >= (grad ? 8 : 12);
+}
+
 }  // namespace fwi

@@ -476,7 +476,7 @@ static fwi_status choose_plan_as(const fwi_plan* P, const fwi_geometry* g, bool 
     out.zc = z_chunk(P, tile_geo(P, out.shape, out.tma, out.x2), vd, grad, sc.pml, B);
   out.S = 1;
   out.res = ResPlan();
-  if (resident) choose_res(P, g, vd, grad, B, sc, &out.res);
+  if (resident) choose_res(P, g, vd, grad, B, K, sc, &out.res);
   if (out.res.on) {
     // (each shot has its own gradient slot)
   } else if (out.tma && P->grid.ndim == 2) {   // the 3D kernels take one shot per CTA

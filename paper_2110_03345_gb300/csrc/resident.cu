@@ -80,10 +80,10 @@ size_t res_buffers(const fwi_plan* P, const fwi_geometry* g, int B) {
 // Tile height: a step takes about t0 + t1 TH (t0: the exchange and the
 // barriers; t1: a row of 128 points on one SM; in units of 18 ns), and B shots
 // take ceil(B / conc) launches of conc shots each.
-void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, int B, const Scheme& sc,
+void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, int B, int K, const Scheme& sc,
                 ResPlan* out) {
   *out = ResPlan();
-  if (!res_eligible(P, grad, B, sc)) return;
+  if (!res_eligible(P, grad, B, sc) || !resident_run(P->nt, K, grad)) return;
   const int gx = (P->L.nx + TILE_X - 1) / TILE_X;
   const int nc = interp_nodes(P->opt.interp, 2);
   double best = 0.0;

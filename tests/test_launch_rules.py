@@ -21,6 +21,8 @@ int main() {
     else if (!strcmp(what, "planes") && read(6))   // nz, columns, density, gradient, PML, most chunks
       printf("%d\n", fwi::z_planes(152, (int)a[0], (long long)a[1], a[2] != 0, a[3] != 0, a[4] != 0, 64,
                                    (long long)a[5]));
+    else if (!strcmp(what, "run") && read(3))
+      printf("%d\n", (int)fwi::resident_run((int)a[0], (int)a[1], a[2] != 0));
     else return 1;
   }
 }
@@ -134,3 +136,20 @@ def test_planes_fit_their_limits(rules):
         else:
             chunks = -(-nz // int(z))
             assert 1 <= z <= 64 and chunks <= most and -(-nz // chunks) == z   # chunks of equal planes
+
+
+# steps between checkpoints of a gradient of 200 (ms), and steps of short runs (gradient or not,
+# us): per-step and resident times, each summed over four grids
+CKPT = [(1, 32.1, 53.0), (2, 22.8, 28.9), (3, 19.2, 21.7), (4, 17.5, 18.1), (6, 16.1, 14.6), (8, 15.2, 12.7),
+        (12, 14.6, 11.0), (24, 13.8, 9.3)]
+SHORT = [(1, 1, 973, 1099), (2, 1, 1032, 1111), (8, 1, 1315, 1256), (16, 1, 1673, 1435), (1, 0, 747, 825),
+         (2, 0, 760, 834), (4, 0, 802, 850), (8, 0, 882, 890), (16, 0, 1020, 968), (32, 0, 1314, 1110)]
+
+
+def test_resident_runs(rules):
+    for (K, per_step, resident), on in zip(CKPT, rules([("run", 201, r[0], 1) for r in CKPT])):
+        assert on == (resident < per_step), K
+    for (steps, grad, per_step, resident), on in zip(SHORT, rules([("run", r[0] + 1, 0, r[1]) for r in SHORT])):
+        assert on == (resident < per_step), (steps, grad)
+    # checkpoints as far apart as the run are none, and they are a gradient's alone
+    assert rules([("run", 9, 8, 1), ("run", 9, 3, 1), ("run", 201, 3, 0)]) == [1, 0, 1]
