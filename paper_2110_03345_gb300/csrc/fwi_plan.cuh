@@ -311,7 +311,8 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc);
 fwi_status choose_plan(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, Plan& out,
                        bool split = false, const Scheme& sc = Scheme());
 constexpr double GROUP_TAIL = 0.55;   // (the PML's: 0.75)
-int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail = GROUP_TAIL);
+int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail = GROUP_TAIL,
+               double* shot_times = nullptr);
 int shot_group(const fwi_plan* P, int shape, int B, const Scheme& sc);
 int z_chunk(const fwi_plan* P, const TileGeo& T, bool vd, bool grad, bool pml, int B);
 void carve_work(fwi_plan* P, const Plan& pl, const fwi_geometry* g, bool vd, Carve& C, Work& W);

@@ -69,4 +69,18 @@ inline bool resident_run(int nt, int K, bool grad) {
   return grad && K > 0 && K < nt - 1 ? K >= 6 : nt - 1 >= (grad ? 8 : 12);
 }
 
+// Whether a resident call beats the per-step kernels: `units` is choose_res's estimate of a
+// resident step (all rounds of shots), `shot_times` shot_group's of a per-step launch.  The
+// estimates in us are fits over nine grids of 256 x 256 - 1024 x 1024 and one to 32 shots
+// (8th order; residuals 8%); within 2% of each other the call stays resident.  Without this
+// a last round of few shots was not seen (resident / per-step, us per step or step pair):
+// 456 x 485 with density, forward of 8, 9 and 10 shots 8.6 / 9.4, 10.5 / 10.2, 12.2 / 10.2; gradient
+// of 12 and 13 shots 30.1 / 31.3, 39.5 / 31.4; 700 x 748 gradient of 6 and 7 29.3 / 32.2, 38.6 / 35.0.
+inline bool resident_pays(double units, double shot_times, bool grad, bool vd) {
+  const double per_step = grad ? (vd ? 4.23 + 3.13 * shot_times : 4.25 + 2.38 * shot_times)
+                               : (vd ? 2.50 + 1.12 * shot_times : 2.73 + 0.89 * shot_times);
+  const double resident = units * (grad ? (vd ? 0.0546 : 0.0418) : (vd ? 0.0234 : 0.0193));
+  return resident <= 1.02 * per_step;
+}
+
 }  // namespace fwi

@@ -383,7 +383,7 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc) {
 // 311.4; fourth-order scheme, 6 shots (800 x 872) 80.6 -> 76.1, 15 shots
 // (1024 x 1024) 246.1 -> 243.8; 6 shots of the PML
 // (1024 x 1024) 106.8 -> 103.9.
-int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail) {
+int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, double tail, double* shot_times) {
   int most = 1, best = 1;
   for (const auto& ts : tiles_shots) most = std::max(most, ts.second);
   double least = 0.0;
@@ -396,6 +396,7 @@ int shot_group(int nsm, const std::vector<std::pair<int, int>>& tiles_shots, dou
       best = S;
     }
   }
+  if (shot_times) *shot_times = least;
   return best;
 }
 

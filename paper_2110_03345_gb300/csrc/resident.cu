@@ -115,6 +115,12 @@ void choose_res(const fwi_plan* P, const fwi_geometry* g, bool vd, bool grad, in
       }
     }
   if (!r.on) return;
+  int id = 0, shape = 0;
+  bool tma = false;
+  double shot_times = 0.0;
+  if (!resolve_tile(P, 0, &id, &shape, &tma)) return;
+  shot_group(P->nsm, {{tile_geo(P, shape, true).ntiles(), B}}, GROUP_TAIL, &shot_times);
+  if (!resident_pays(best, shot_times, grad, vd)) return;
   int nval = 0;
   for (int s = 0; s < g->nshots; ++s)
     nval = std::max(nval, most_entries(P, g->src_xyz + (size_t)s * g->nsrc * 2, g->nsrc, r.TH, r.gx, r.gy));

@@ -23,6 +23,8 @@ int main() {
                                    (long long)a[5]));
     else if (!strcmp(what, "run") && read(3))
       printf("%d\n", (int)fwi::resident_run((int)a[0], (int)a[1], a[2] != 0));
+    else if (!strcmp(what, "resident") && read(4))
+      printf("%d\n", (int)fwi::resident_pays(a[0], a[1], a[2] != 0, a[3] != 0));
     else return 1;
   }
 }
@@ -136,6 +138,81 @@ def test_planes_fit_their_limits(rules):
         else:
             chunks = -(-nz // int(z))
             assert 1 <= z <= 64 and chunks <= most and -(-nz // chunks) == z   # chunks of equal planes
+
+
+# gradient, density, shots, units, shot times, us per step (pair) per-step and resident, of 256 x
+# 256, 456 x 485, 700 x 748, 800 x 872 and 1024 x 1024 points
+RESIDENT = """
+0 1 24 312.8 5.439 8.87 7.77
+0 1 32 386.8 6.703 10.14 9.13
+0 0 24 312.8 5.439 7.98 6.66
+0 0 32 386.8 6.703 8.67 7.51
+1 1 32 386.8 6.703 26.27 22.68
+1 0 32 386.8 6.703 21.43 17.66
+0 1 6 298 5.084 8.39 7.35
+0 1 7 342.4 5.847 8.63 8.56
+0 1 8 342.4 6.229 9.41 8.56
+0 1 9 447 6.779 10.24 10.46
+0 1 10 513.6 7.374 10.23 12.2
+0 0 6 298 5.084 7.37 6.3
+0 0 7 342.4 5.847 7.74 7.03
+0 0 8 342.4 6.229 8.25 7.02
+0 0 9 447 6.779 9.04 8.97
+0 0 10 513.6 7.374 8.74 10.16
+1 1 9 447 6.779 26.2 24.71
+1 1 10 513.6 7.374 25.49 30.06
+1 1 11 513.6 7.924 29.12 30.03
+1 1 12 513.6 8.305 31.28 30.08
+1 1 13 684.8 9.068 31.42 39.45
+1 1 14 684.8 9.450 31.59 39.43
+1 1 15 684.8 9.832 33.06 39.51
+1 1 16 684.8 10.382 38.83 39.3
+1 0 9 447 6.779 21.27 19.68
+1 0 10 513.6 7.374 20.68 22.58
+1 0 11 513.6 7.924 22.59 22.46
+1 0 12 513.6 8.305 24.77 22.06
+1 0 13 684.8 9.068 24.89 29.41
+1 0 14 684.8 9.450 25.08 29.11
+1 0 15 684.8 9.832 26.64 29.04
+1 0 16 684.8 10.382 30.69 29.23
+0 1 3 372 5.674 8.44 8.53
+0 1 4 372 6.861 10.26 8.69
+0 0 3 372 5.674 7.3 7.23
+0 0 4 372 6.861 8.71 7.24
+1 1 4 372 6.861 24.83 20.19
+1 1 5 558 8.279 27.55 29.3
+1 1 6 558 9.147 32.15 29.33
+1 1 7 744 10.566 35 38.61
+1 0 4 372 6.861 19.74 15.76
+1 0 5 558 8.279 21.87 23.15
+1 0 6 558 9.147 25.24 22.99
+1 0 7 744 10.566 27.6 29.96
+0 1 2 298 5.104 8.53 7.61
+0 1 3 447 6.805 10.29 10.62
+0 0 2 298 5.104 7.1 6.24
+0 0 3 447 6.805 8.95 8.8
+1 1 3 447 6.805 25.93 23.81
+1 1 4 596 8.507 31.69 31.09
+1 1 5 745 10.208 37.44 38.37
+1 0 3 447 6.805 20.66 19.16
+1 0 4 596 8.507 25.22 25.34
+1 0 5 745 10.208 29.69 31.33
+0 1 2 357.2 6.703 10.14 8.94
+0 0 2 357.2 6.703 8.25 7.22
+1 1 2 357.2 6.703 24.39 20.16
+1 1 3 535.8 8.937 31.59 29
+1 0 2 357.2 6.703 19.11 15.56
+1 0 3 535.8 8.937 24.53 22.58
+"""
+
+
+def test_resident_or_per_step(rules):
+    table = [list(map(float, line.split())) for line in RESIDENT.strip().splitlines()]
+    picks = rules([("resident", u, s, int(g), int(d)) for g, d, _, u, s, _, _ in table])
+    assert 0 < sum(picks) < len(picks)
+    for row, on in zip(table, picks):
+        per_step, resident = row[5:]
+        assert resident <= 1.1 * per_step if on else per_step <= 1.05 * resident, row
 
 
 # steps between checkpoints of a gradient of 200 (ms), and steps of short runs (gradient or not,
