@@ -659,11 +659,16 @@ fwi_status fwi_plan_estimate(const fwi_plan* plan, const fwi_geometry* geom, int
                              size_t* bytes) {
   if (!plan || !bytes) return fail(FWI_ERR_INVALID_ARG, "NULL argument");
   FWI_TRY(validate_geometry(plan, geom));
-  Plan pl;
   Scheme sc;
   FWI_TRY(resolve_scheme(plan, nullptr, &sc));
-  FWI_TRY(choose_plan(plan, geom, true, gradient != 0, pl, false, sc));
-  *bytes = pl.bytes + tables_bound(plan, geom, pl) * 2;
+  // with density and without: a call without may run resident where one with does not, and
+  // must find room for it in a budget of these bytes
+  *bytes = 0;
+  for (bool vd : {true, false}) {
+    Plan pl;
+    FWI_TRY(choose_plan(plan, geom, vd, gradient != 0, pl, false, sc));
+    *bytes = std::max(*bytes, pl.bytes + tables_bound(plan, geom, pl) * 2);
+  }
   return FWI_OK;
 }
 
