@@ -11,14 +11,15 @@ namespace fwi {
 // x 180 x 200, 160 at 256^3 and 320-430 at 384^3.  Small launches are bound by latency, not
 // by the loads and the arithmetic that the flags spare, and lose to the choice per plane.
 // Gain per step (step pair for gradients) with a density that is constant within two
-// tissues, order 10, in us: leapfrog forward 100^3 -0.4, 128^3 -0.2, 152 x 160 x 176 0, 192
-// x 180 x 200 2.5, 256^3 8.4, 384^3 53; gradient -1.8, -1.3, -0.4, 11.8, 20.6, 118, four shots
-// of 300 x 64 x 64 6.7; PML forward 64^3 0, 100^3 0.6, 300 x 64 x 64 2.2, 128^3 4.2, 256^3 17;
-// gradient 0, 2.3, 5.8, 5.9, 56.  So the leapfrog takes them from 4.5 million points, the
-// PML from a million, and either where the run is long enough to win their cost back
-// (8-37 steps).
+// tissues, order 10, in us: leapfrog forward 100^3 -0.4, 128^3 -0.2, 150^3 -0.2, 152 x 160 x
+// 176 0, 130 x 226 x 143 3, 192 x 180 x 200 2.5, 256^3 8.4, 384^3 53; gradient -1.8, -1.3, 2.6,
+// -0.4, 12, 11.8, 20.6, 118, four shots of 300 x 64 x 64 6.7; PML forward 64^3 0, 100^3 0.6,
+// 300 x 64 x 64 2.2, 128^3 4.2, 256^3 17; gradient 0, 2.3, 5.8, 5.9, 56.  So the leapfrog takes
+// them from three million points, the PML from a million, and either where the run is long
+// enough to win their cost back.
 inline bool density_flags_pay(long long points, int nt, bool grad, bool pml) {
-  return points >= (pml ? 1000000LL : 4500000LL) && (grad ? 4LL : 1LL) * nt >= 40;
+  return points >= (pml ? 1000000LL : 3000000LL) &&
+         (grad ? 4LL : 1LL) * nt >= (points >= 6000000LL ? 40 : pml ? 60 : 160);
 }
 
 // Planes per CTA of the default 3D variant (0: none fits `most_chunks`), for `cols` column

@@ -1,4 +1,4 @@
-"""Calls whose grid points over all slots are enough for the density flags (4.5 million, the
+"""Calls whose grid points over all slots are enough for the density flags (three million, the
 PML a million) against the same shots one at a time, whose launches add every density
 term: what the flags leave out are zeros, so traces and misfits are equal, and gradients
 to the order in which the shots are summed (32 terms of 6e-8 each add up as their root:
@@ -19,7 +19,7 @@ def test_flags_against_every_term(scheme, order, shots):
     shape, nt, dx = (45, 30, 131), 44, 0.5e-3
     p = inputs.skull_problem(shape, dx, nt, nrec=64, every=1, order=order, nb=5, f0=250e3)
     src = p.src_xyz[:shots]
-    assert len(src) == shots and np.prod(shape) * shots >= (1e6 if scheme == "pml" else 4.5e6)
+    assert len(src) == shots and np.prod(shape) * shots >= (1e6 if scheme == "pml" else 3e6)
     geo = binding.Geometry(src, p.rec_xyz)
     vp = to_dev(p.vp)
     w = to_dev(np.broadcast_to(np.asarray(p.wavelet)[:1, :1], (shots, 1, nt)))

@@ -44,31 +44,44 @@ def rules(tmp_path_factory):
     return ask
 
 
-# grid, PML, forward: cost of the flags and gain per step, gradient: the same (us)
-FLAGS = [((40, 44, 48), 0, 39.2, 0.12, 53.4, -0.04), ((64, 64, 64), 0, 40.0, -0.60, 51.8, -0.49),
-         ((100, 100, 100), 0, 53.2, -0.38, 58.8, -1.82), ((128, 128, 128), 0, 50.7, -0.19, 61.7, -1.30),
-         ((152, 160, 176), 0, 65.1, -0.05, 78.1, -0.40), ((300, 64, 64), 0, 41.5, 0.15, 45.9, 1.11),
-         ((192, 180, 200), 0, 91.7, 2.48, 97.6, 11.78), ((256, 256, 256), 0, 163.3, 8.44, 163.8, 20.56),
-         ((384, 384, 384), 0, 426.3, 52.66, 315.5, 118.27), ((64, 64, 64), 1, 45.3, -0.19, 50.0, -0.12),
-         ((128, 128, 128), 1, 43.8, 4.24, 52.7, 5.90), ((152, 160, 176), 1, 70.2, 5.75, 70.2, 7.62),
-         ((300, 64, 64), 1, 32.8, 2.25, 40.8, 5.75), ((192, 180, 200), 1, 88.7, 11.59, 70.2, 40.70),
-         ((256, 256, 256), 1, 153.2, 17.46, 122.1, 55.66), ((384, 384, 384), 1, 425.9, 59.39, 250.8, 240.87)]
+# grid, PML, forward: cost of the flags, gain per step and time of a step without them, gradient:
+# the same (us)
+FLAGS = [
+    ((40, 44, 48), 0, 39.2, 0.12, 10, 53.4, -0.04, 25.4),
+    ((64, 64, 64), 0, 40, -0.6, 10.9, 51.8, -0.49, 27.1),
+    ((64, 64, 64), 1, 45.3, -0.19, 39.5, 50, -0.12, 79.8),
+    ((100, 100, 100), 0, 53.2, -0.38, 15.7, 58.8, -1.82, 36.7),
+    ((100, 100, 100), 1, 49.4, 0.64, 57.4, 56, 2.28, 115.2),
+    ((128, 128, 128), 0, 50.7, -0.19, 18.7, 61.7, -1.3, 50.8),
+    ((128, 128, 128), 1, 43.8, 4.24, 80.4, 52.7, 5.9, 173.6),
+    ((152, 160, 176), 0, 65.1, -0.05, 38.2, 78.1, -0.4, 102.9),
+    ((152, 160, 176), 1, 70.2, 5.75, 161.1, 70.2, 7.62, 339.5),
+    ((192, 180, 200), 0, 91.7, 2.48, 75.3, 97.6, 11.78, 167.2),
+    ((192, 180, 200), 1, 88.7, 11.59, 307.2, 70.2, 40.7, 520.5),
+    ((256, 256, 256), 0, 163.3, 8.44, 112, 163.8, 20.56, 278.5),
+    ((256, 256, 256), 1, 153.2, 17.46, 373.8, 122.1, 55.66, 866.4),
+    ((384, 384, 384), 0, 426.3, 52.66, 363.4, 315.5, 118.27, 886.5),
+    ((384, 384, 384), 1, 425.9, 59.39, 999.7, 250.8, 240.87, 2487.2),
+    ((300, 64, 64), 0, 41.5, 0.15, 15.2, 45.9, 1.11, 31.6),
+    ((300, 64, 64), 1, 32.8, 2.25, 42.8, 40.8, 5.75, 91.3),
+]
 
 
 def test_density_flags(rules):
-    """Where the flags are made they win more than they cost, and no call of hundreds of
-    steps on a large grid goes without them."""
+    """Where the flags are made they win their cost, or lose 2.5% of the call at most, and no
+    call of a hundred steps on a large grid goes without them."""
     rows, want = [], []
-    for shape, pml, fc, fg, gc, gg in FLAGS:
-        for grad, cost, gain in ((0, fc, fg), (1, gc, gg)):
-            for nt in (2, 3, 9, 10, 20, 40, 41, 100, 1000):
-                rows.append(("flags", shape[0] * shape[1] * shape[2], nt, grad, pml))
-                want.append((gain * nt - cost, nt, shape[0] * shape[1] * shape[2] > 5e6))
-    for r, on, (net, nt, large) in zip(rows, rules(rows), want):
+    for shape, pml, fc, fg, fs, gc, gg, gs in FLAGS:
+        n = shape[0] * shape[1] * shape[2]
+        for grad, cost, gain, step in ((0, fc, fg, fs), (1, gc, gg, gs)):
+            for nt in (2, 3, 9, 10, 15, 20, 30, 40, 60, 100, 160, 1000):
+                rows.append(("flags", n, nt, grad, pml))
+                want.append((gain * nt - cost, nt, step, n > 4e6))
+    for r, on, (net, nt, step, large) in zip(rows, rules(rows), want):
         if on:
-            assert net > -20, r
+            assert net >= -0.025 * nt * step, r
         else:
-            assert not (large and nt >= 100), r
+            assert not (large and nt >= 160), r
 
 
 # us per step (pair) of one shot by planes per CTA, order 10: leapfrog with density (leap) and
