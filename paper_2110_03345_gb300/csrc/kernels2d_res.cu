@@ -34,8 +34,11 @@
 // shared data pipe is busy 56% of the time and the FMA pipe 40% at 14 warps of
 // 128 registers; every CTA keeps step with the slowest, so a step costs the
 // slowest tile's arithmetic plus about 1200 cycles of exchange and barriers.
-// A step takes 1.35 us at 256 x 256 (per-step launches 3.5), 2.6 at 700 x 748
-// (4.1) and 3.9 at 1024 x 1024 (5.9); an adjoint step 4.9 there (10.8).
+// One shot, 64 receivers, 8th order, time of a call of 1000 steps per step, per-step kernels
+// -> resident, forward / forward and adjoint with imaging, in us: 256 x 256 with density
+// 3.6 -> 2.0 / 8.0 -> 4.2, without 3.5 -> 1.7 / 7.2 -> 3.7; 700 x 748 with 4.0 -> 2.7 / 9.1 -> 7.5,
+// without 3.9 -> 2.4 / 8.3 -> 5.4; 1024 x 1024 with 5.7 -> 3.7 / 15.2 -> 9.1, without 5.1 -> 3.2 /
+// 12.4 -> 7.0.
 // Tried and slower: 28 warps of 72 registers with one row each (shared loads
 // and spills), four rows in one phase (the exchange is exposed), scalar
 // weights in place of packed ones, the outer columns sent by every warp.
@@ -579,7 +582,9 @@ __global__ void __launch_bounds__(32 * RES_WARPS, 1) k_res2d(const ResParams p) 
   // A launch of one step has received nothing yet: wait for the neighbours' words,
   // so that no tile is written back before its neighbours have read it (a word is
   // sent after its tile is staged).  Each thread waits for its own cells only, hence
-  // the barrier; longer launches have passed one behind the receive of their steps.
+  // the barrier; longer launches have passed one behind the receive of their steps.  (On
+  // time-out the flag makes the call an error; an early return here cost one instantiation
+  // 5% of its step.)
   if (p.steps == 1) {
     bool ok = true;
     if (PH == 2) {
@@ -588,11 +593,8 @@ __global__ void __launch_bounds__(32 * RES_WARPS, 1) k_res2d(const ResParams p) 
     }
 #pragma unroll
     for (int ph = 0; ph < PH; ++ph) ok = receive(ph, s_u1, 1u, p.tag0 + 1, ahead, false) && ok;
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0 && p.flags) atomicOr(p.flags, 2);
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      return;
-    }
+    if (!ok && p.flags) atomicOr(p.flags, 2);
+    __syncthreads();
   }
   // ---- state back to global memory: u^{n+steps} and u^{n+steps-1}
   const float4* fu = (p.steps & 1) ? s_u1 : s_u0;

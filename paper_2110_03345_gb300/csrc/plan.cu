@@ -373,9 +373,12 @@ fwi_status resolve_scheme(const fwi_plan* P, const fwi_model* m, Scheme* sc) {
 // Shots per CTA (S) of a 2D per-step launch over problems of (tiles, shots).  In
 // shot times, a CTA of S shots takes about S + 1 (the model loads and the gradient
 // update cost one), two CTAs per SM work at a time, and `tail` of a CTA is waited
-// for at the end of the step: about half, more with the PML, whose CTAs differ (its
-// 1024 x 1024 gradient of 6 shots: S = 3 27.3 ms, S = 6 29.0 ms).  The S with the least
-// of the sum is taken.
+// for at the end of a launch: about half, more with the PML, whose step pair has four launches
+// (us per gradient step pair with tails 0.75 / 0.55 where they differ,
+// with density: 300 x 320, 6 and 8 shots 40.4 / 45.7 and 44.6 / 47.8; 600 x 640, 3, 8 and 12
+// shots 43.9 / 49.9, 73.0 / 73.4 and 97.1 / 99.7; 800 x 872, 4 and 16 shots 64.8 / 71.4 and
+// 185.3 / 191.4; 1024 x 1024, 6 shots 111.0 / 110.6; of 84 calls of six grids none is slower by
+// more than that).  The S with the least of the sum is taken.
 // Measured against the largest S <= 6 that leaves four waves of CTAs, us per
 // gradient step pair (8th order, density): 456 x 485, 16 shots 50.8 -> 39.8; 700 x
 // 748, 6 shots 43.3 -> 32.8, 10 shots 70.0 -> 47.9; 1024 x 1024, 6 shots 62.9 ->

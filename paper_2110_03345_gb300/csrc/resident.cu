@@ -38,15 +38,11 @@ int most_entries(const fwi_plan* P, const double* xyz, long long n, int TH, int 
 
 // Whether a call of B shots may run resident.  A resident shot costs the same
 // whatever the number of shots; the per-step kernels' cost per shot falls as CTAs
-// of several shots fill the SMs.  Measured on a GB300 in us per step (per step pair
-// for gradients), per-step -> resident, 8th order with density: 256 x 256, one shot
-// 4.1 -> 2.3 forward and 9.1 -> 4.6 gradient; 700 x 748, two shots 5.9 -> 4.2 and
-// 14.7 -> 10.2; 1024 x 1024, one shot 5.9 -> 4.4 and 16.6 -> 10.5.  Forward runs
-// break even at about 8 tile-shots (128 x 16 points) per SM (456 x 485, twelve
-// shots 9.2 -> 9.3; 700 x 748, four 8.9 -> 7.9, six 11.7 -> 11.8; 1024 x 1024, two
-// 8.6 -> 8.2, three 11.3 -> 11.9), gradients at about 12.5 (456 x 485, 16 shots 29.1 ->
-// 28.5, twenty 32.6 -> 35.4; 700 x 748, six 31.3 -> 29.7, eight 38.5 -> 39.5; 1024 x
-// 1024, three 30.7 -> 29.9, four 38.2 -> 39.1).
+// of several shots fill the SMs (one and two shots: the figures of kernels2d_res.cu;
+// two shots of 1024 x 1024 with density 8.4 -> 7.1 us per forward step and 22.0 -> 18.0 per
+// step pair).  Above 8 tile-shots (128 x 16 points) per SM for forward runs and 12.5 for
+// gradients the per-step kernels are as good in most calls (per-step / resident there
+// 0.77 - 1.14); below, choose_res compares the two (resident_pays).
 bool res_eligible(const fwi_plan* P, bool grad, int B, const Scheme& sc) {
   if (P->grid.ndim != 2 || sc.ext() || P->fixed_memory || P->per_step || P->opt.tile != 0 ||
       P->opt.shots_per_cta != 0 || B < 1 || P->nt < 2)
